@@ -37,10 +37,10 @@
  *   launched.  Errors found on the device (non-finite values, bad flags) are
  *   sticky in the grid's status word and reported by ocp_get_status().
  * There is no CPU fallback: every compute call runs CUDA kernels for sm_103a.
- * Only ocp_grid_create, ocp_batch_create, their destroy calls and the first
- *   ocp_linearize_pn on a grid (its phase-split data) allocate or free device
- *   memory; the first ocp_bicgstab* call on a grid creates a stream and a
- *   CUDA graph that the grid keeps.
+ * Only ocp_grid_create, ocp_batch_create, their destroy calls, the first
+ *   ocp_linearize_pn on a grid (its phase-split data) and the first
+ *   ocp_bicgstab* of each block size (the solver's copy of the scaled matrix)
+ *   allocate or free device memory.
  * ocp_last_error() returns a thread-local message describing the last failure.
  */
 #ifndef OCP_H
@@ -303,14 +303,14 @@ int64_t ocp_solver_work_doubles(const ocp_grid* grid);
  * scaled cell by cell into the units of the unknowns.  x holds the initial guess
  * on entry and the solution on return; b and x are block-interleaved [nb*N]
  * device vectors; work is a device buffer of ocp_solver_work_doubles().
- * The iterations run as replays of a CUDA graph of eight iterations with the
- * convergence test on the device; the stream is synchronised once per replay.
- * The graph is captured on the first call and kept on the grid while the
- * same bsr_val, x, work (and well terms) are passed; calls on one grid must
- * not overlap from several host threads.  The paper solves with
- * CPR-preconditioned FGMRES in PETSc/Hypre (Sec. 5.1); this plain Krylov
- * solver serves the Newton, adjoint and test drivers.  Returns
- * OCP_ERR_TIMEOUT when maxit is reached, OCP_ERR_NONFINITE on breakdown;
+ * The iterations run in one cooperative launch with the convergence test on
+ * the device; the stream is synchronised once, at the end.  The grid keeps the
+ * solver's copy of D^-1 A (6 nb^2 doubles per cell, 6 for a scalar system),
+ * allocated by the first call; where it does not fit, the same iteration runs
+ * from bsr_val itself.  Calls on one grid must not overlap from several host
+ * threads.  The paper solves with CPR-preconditioned FGMRES in PETSc/Hypre
+ * (Sec. 5.1); this plain Krylov solver serves the Newton, adjoint and test
+ * drivers.  Returns OCP_ERR_TIMEOUT when maxit is reached, OCP_ERR_NONFINITE on breakdown;
  * *iters and *relres (may be NULL) report the final state. */
 ocp_status ocp_bicgstab(ocp_grid* grid, const double* bsr_val, const double* b, double* x, double rtol,
                         int maxit, int transpose, double* work, int* iters, double* relres, void* cuda_stream);

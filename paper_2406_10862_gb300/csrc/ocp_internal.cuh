@@ -139,9 +139,10 @@ struct ocp_grid {
   unsigned* d_sync;          // ordered launch: item counter, then cell and face flags per 32-cell tile
   double* d_pn;              // per-cell data of the (P, N) path, allocated on its first use
   int8_t* d_pn_flag;
-  cudaStream_t solve_cap;    // private stream on which the solver's iterations are captured
-  cudaGraphExec_t solve_exec;  // a block of solver iterations, valid for the buffers in solve_key
-  const void* solve_key[8];
+  void* d_solve_sync;        // the solver's results and barrier slots, allocated by the first solve
+  unsigned long long solve_epoch;   // number of the last barrier of the solves so far
+  double* d_planes;          // its scaled off-diagonal blocks (null where they did not fit)
+  int64_t planes_doubles;
   int64_t scratch_doubles;
   ocp::LaunchCfg cfg;        // launch shape of the linearisation
   int sms;                   // SM count of the device

@@ -5,8 +5,8 @@
 // spmv_grid_t_kernel the transposed product: every output row gathers the
 //                   blocks (n, c) of its column, located in closed form, so
 //                   that it is owned by one thread and no atomics are needed;
-// spmv_bulk_kernel  y = alpha A x + beta y for 2x2 and 1x1 blocks with the
-//                   matrix slices staged by bulk asynchronous copies;
+// spmv_bulk_kernel  y = alpha A x + beta y for 2x2 blocks with the matrix
+//                   slices staged by bulk asynchronous copies;
 // vjp_kernel        lambda^T dR/d(u_new, u_old, ln k, phi) of the residual of
 //                   eqs. 1, 2 and 4: J^T lambda with the column's blocks found in closed form, the
 //                   transmissibility and well-index terms from the stored face
@@ -99,12 +99,11 @@ template <int NB>
 __global__ void __launch_bounds__(kSpmvThreads, kSpmvMinBlocks) spmv_grid_kernel(Params P, const int32_t* __restrict__ row_ptr,
                                                         const double* __restrict__ val, double alpha,
                                                         const double* __restrict__ x, double beta,
-                                                        double* __restrict__ y, int mode,
-                                                        const double* __restrict__ skip) {
+                                                        double* __restrict__ y, int mode) {
   constexpr int B2 = NB * NB;
   pdl_wait();
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (c >= P.N || (skip != nullptr && *skip != 0.0)) return;
+  if (c >= P.N) return;
   int ci, cj, ck;
   cell_ijk(P, c, ci, cj, ck);
   const bool has[7] = {ck > 0, cj > 0, ci > 0, true, ci + 1 < P.nx, cj + 1 < P.ny, ck + 1 < P.nz};
@@ -158,12 +157,11 @@ __global__ void __launch_bounds__(kSpmvThreads, kSpmvMinBlocks) spmv_grid_kernel
 template <int NB>
 __global__ void __launch_bounds__(kSpmvThreads) spmv_grid_t_kernel(Params P, const double* __restrict__ val,
                                                                    double alpha, const double* __restrict__ x,
-                                                                   double beta, double* __restrict__ y, int mode,
-                                                                   const double* __restrict__ skip) {
+                                                                   double beta, double* __restrict__ y, int mode) {
   constexpr int B2 = NB * NB;
   pdl_wait();
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (c >= P.N || (skip != nullptr && *skip != 0.0)) return;
+  if (c >= P.N) return;
   int ci, cj, ck;
   cell_ijk(P, c, ci, cj, ck);
   const bool has[7] = {ck > 0, cj > 0, ci > 0, true, ci + 1 < P.nx, cj + 1 < P.ny, ck + 1 < P.nz};
@@ -198,7 +196,7 @@ __global__ void __launch_bounds__(kSpmvThreads) spmv_grid_t_kernel(Params P, con
   }
 }
 
-// Product for 2x2 and 1x1 blocks with the CTA's slice of the matrix staged
+// Product for 2x2 blocks with the CTA's slice of the matrix staged
 // in shared memory by one bulk asynchronous copy (the TMA unit), completing
 // on an mbarrier while the CTA's threads gather their x entries.  Rows of a
 // CTA are consecutive, so their blocks are one contiguous range of `val`.
@@ -241,11 +239,10 @@ __global__ void __launch_bounds__(kBulkRows) spmv_bulk_kernel(Params P, const in
                                                               long long nnzb, const double* __restrict__ val,
                                                               double alpha, const double* __restrict__ x,
                                                               double beta, double* __restrict__ y, int mode,
-                                                              int* __restrict__ status, const double* __restrict__ skip) {
+                                                              int* __restrict__ status) {
   constexpr int B2 = NB * NB;
   constexpr long long BB = 8 * B2;
   pdl_wait();
-  if (skip != nullptr && *skip != 0.0) return;     // the same for every thread: before any barrier
   extern __shared__ __align__(128) unsigned char sbuf[];
   __shared__ __align__(8) unsigned long long bar;
   const long long r0 = (long long)blockIdx.x * kBulkRows;
@@ -494,31 +491,24 @@ cudaError_t launch_setup(ocp_grid* g, const double* d_lnk, double dx, double dy,
 }
 
 cudaError_t launch_spmv(const ocp_grid* g, const double* val, double alpha, const double* x, double beta,
-                        double* y, int transpose, cudaStream_t s, int nbs, const double* skip) {
+                        double* y, int transpose, cudaStream_t s) {
   const long long N = g->prm.N;
   const int mode = (beta != 0.0) ? 2 : (alpha != 1.0 ? 1 : 0);
   const unsigned gblocks = (unsigned)((N + kSpmvThreads - 1) / kSpmvThreads);
-  const int nb = nbs > 0 ? nbs : g->prm.nb;
-  // 2x2 and 1x1 products stage their matrix slices by bulk copy when the
-  // matrix is 16-byte aligned (the copy's rule); otherwise, and for 3x3, the
-  // register kernel runs.  Both give identical bits.  Every product is a
-  // programmatic launch (launch_pdl): it is scheduled while the kernel before
-  // it finishes and waits for it before touching memory.
+  // 2x2 products stage their matrix slices by bulk copy when the matrix is
+  // 16-byte aligned (the copy's rule); otherwise, and for 3x3, the register
+  // kernel runs.  Both give identical bits.  Every product is a programmatic
+  // launch (launch_pdl): it is scheduled while the kernel before it finishes
+  // and waits for it before touching memory.
   const bool bulk = ((uintptr_t)val & 15) == 0;
   const unsigned bblocks = (unsigned)((N + kBulkRows - 1) / kBulkRows);
-  if (nb == 3) {
-    if (transpose) return launch_pdl(spmv_grid_t_kernel<3>, gblocks, kSpmvThreads, 0, s, g->prm, val, alpha, x, beta, y, mode, skip);
-    return launch_pdl(spmv_grid_kernel<3>, gblocks, kSpmvThreads, 0, s, g->prm, (const int32_t*)g->d_row_ptr, val, alpha, x, beta, y, mode, skip);
-  } else if (nb == 2) {
-    if (transpose) return launch_pdl(spmv_grid_t_kernel<2>, gblocks, kSpmvThreads, 0, s, g->prm, val, alpha, x, beta, y, mode, skip);
-    if (bulk) return launch_pdl(spmv_bulk_kernel<2>, bblocks, kBulkRows, bulk_smem_bytes<2>(), s, g->prm, (const int32_t*)g->d_row_ptr, (long long)g->nnzb, val, alpha, x, beta, y, mode, g->d_status, skip);
-    return launch_pdl(spmv_grid_kernel<2>, gblocks, kSpmvThreads, 0, s, g->prm, (const int32_t*)g->d_row_ptr, val, alpha, x, beta, y, mode, skip);
-  } else {
-    if (transpose) return launch_pdl(spmv_grid_t_kernel<1>, gblocks, kSpmvThreads, 0, s, g->prm, val, alpha, x, beta, y, mode, skip);
-    if (bulk) return launch_pdl(spmv_bulk_kernel<1>, bblocks, kBulkRows, bulk_smem_bytes<1>(), s, g->prm, (const int32_t*)g->d_row_ptr, (long long)g->nnzb, val, alpha, x, beta, y, mode, g->d_status, skip);
-    return launch_pdl(spmv_grid_kernel<1>, gblocks, kSpmvThreads, 0, s, g->prm, (const int32_t*)g->d_row_ptr, val, alpha, x, beta, y, mode, skip);
+  if (g->prm.nb == 3) {
+    if (transpose) return launch_pdl(spmv_grid_t_kernel<3>, gblocks, kSpmvThreads, 0, s, g->prm, val, alpha, x, beta, y, mode);
+    return launch_pdl(spmv_grid_kernel<3>, gblocks, kSpmvThreads, 0, s, g->prm, (const int32_t*)g->d_row_ptr, val, alpha, x, beta, y, mode);
   }
-  return cudaGetLastError();
+  if (transpose) return launch_pdl(spmv_grid_t_kernel<2>, gblocks, kSpmvThreads, 0, s, g->prm, val, alpha, x, beta, y, mode);
+  if (bulk) return launch_pdl(spmv_bulk_kernel<2>, bblocks, kBulkRows, bulk_smem_bytes<2>(), s, g->prm, (const int32_t*)g->d_row_ptr, (long long)g->nnzb, val, alpha, x, beta, y, mode, g->d_status);
+  return launch_pdl(spmv_grid_kernel<2>, gblocks, kSpmvThreads, 0, s, g->prm, (const int32_t*)g->d_row_ptr, val, alpha, x, beta, y, mode);
 }
 
 cudaError_t launch_vjp(const ocp_grid* g, const double* u_new, const int8_t* f_new, const double* u_old,

@@ -7,10 +7,10 @@
 //                     B = dR_cell/dp_bh per perforation, the well equation
 //                     (pressure or surface-rate control) R_w, C = dR_w/du_cell
 //                     per perforation and D = dR_w/dp_bh;
-//   schur_kernel      one warp per well: the Schur complement of the well
-//                     unknowns, applied matrix-free next to the block-CSR
-//                     SpMV -- (A - B D^-1 C) x, the reduced right-hand side
-//                     and the back-substitution for the well unknowns;
+//   schur_kernel      one warp per well: the reduced right-hand side of the
+//                     system without the well unknowns (the solver applies
+//                     its Schur complement A - B D^-1 C, krylov.cu) and the
+//                     back-substitution for the well unknowns;
 //   well_update_kernel  p_bh update and the switch of a rate-controlled well
 //                     to pressure control at its limit;
 //   cnv_kernel        scaled residual maxima for the Newton convergence test.
@@ -104,39 +104,35 @@ __global__ void __launch_bounds__(kWellThreads) well_rows_kernel(
   }
 }
 
-// MODE 0: out += alpha Bs (D^-1 (Cs . in));  MODE 1: out += alpha Bs (D^-1 bw);
-// MODE 2: xw = D^-1 (bw - Cs . in).
-template <int NB, int MODE>
+// REDUCE: out -= Bs (D^-1 bw) (the right-hand side of the eliminated system);
+// else xw = D^-1 (bw - Cs . in).
+template <int NB, bool REDUCE>
 __global__ void __launch_bounds__(kWellThreads) schur_kernel(const Perf* __restrict__ perf,
                                                              const int32_t* __restrict__ first, int nwell,
-                                                             WellSchur ws, double alpha,
-                                                             const double* __restrict__ in, double* out,
-                                                             const double* __restrict__ bw, double* __restrict__ xw,
-                                                             const double* __restrict__ skip) {
+                                                             WellSchur ws, const double* __restrict__ in, double* out,
+                                                             const double* __restrict__ bw, double* __restrict__ xw) {
   const int w = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
-  if (w >= nwell || (skip != nullptr && *skip != 0.0)) return;
+  if (w >= nwell) return;
   const int k0 = first[w], k1 = first[w + 1];
-  double t = 0.0;
-  if (MODE != 1) {
+  const double dw = ws.d[w];
+  if (REDUCE) {
+    const double tw = -(bw[w] / dw);
     for (int k = k0 + lane; k < k1; k += 32) {
       const long long c = perf[k].cell;
 #pragma unroll
-      for (int v = 0; v < NB; ++v) t = fma(ws.cs[(long long)k * NB + v], in[c * NB + v], t);
+      for (int e = 0; e < NB; ++e) out[c * NB + e] = fma(ws.bs[(long long)k * NB + e], tw, out[c * NB + e]);
     }
-    t = warp_sum(t);
-  }
-  const double dw = ws.d[w];
-  if (MODE == 2) {
-    if (lane == 0) xw[w] = (bw[w] - t) / dw;
     return;
   }
-  const double tw = alpha * ((MODE == 1 ? bw[w] : t) / dw);
+  double t = 0.0;
   for (int k = k0 + lane; k < k1; k += 32) {
     const long long c = perf[k].cell;
 #pragma unroll
-    for (int e = 0; e < NB; ++e) out[c * NB + e] = fma(ws.bs[(long long)k * NB + e], tw, out[c * NB + e]);
+    for (int v = 0; v < NB; ++v) t = fma(ws.cs[(long long)k * NB + v], in[c * NB + v], t);
   }
+  t = warp_sum(t);
+  if (lane == 0) xw[w] = (bw[w] - t) / dw;
 }
 
 __global__ void well_update_kernel(int nwell, const Perf* __restrict__ perf, const int32_t* __restrict__ first,
@@ -211,18 +207,25 @@ struct Guard {
 
 }  // namespace
 
-cudaError_t launch_well_schur(const ocp_grid* g, const WellSchur& ws, int mode, double alpha, const double* in,
-                              double* out, const double* bw, double* xw, cudaStream_t s, const double* skip) {
+cudaError_t launch_well_reduce(const ocp_grid* g, const WellSchur& ws, const double* bw, double* out,
+                               cudaStream_t s) {
   if (g->nwell == 0) return cudaSuccess;
   const unsigned nb = well_blocks(g->nwell);
-  const bool three = g->prm.nb == 3;
-#define OCP_SCHUR(NBV, M) \
-  schur_kernel<NBV, M><<<nb, kWellThreads, 0, s>>>(g->d_perf, g->d_well_first, g->nwell, ws, alpha, in, out, bw, xw, \
-                                                    skip)
-  if (mode == 0) { if (three) OCP_SCHUR(3, 0); else OCP_SCHUR(2, 0); }
-  else if (mode == 1) { if (three) OCP_SCHUR(3, 1); else OCP_SCHUR(2, 1); }
-  else { if (three) OCP_SCHUR(3, 2); else OCP_SCHUR(2, 2); }
-#undef OCP_SCHUR
+  if (g->prm.nb == 3)
+    schur_kernel<3, true><<<nb, kWellThreads, 0, s>>>(g->d_perf, g->d_well_first, g->nwell, ws, nullptr, out, bw, nullptr);
+  else
+    schur_kernel<2, true><<<nb, kWellThreads, 0, s>>>(g->d_perf, g->d_well_first, g->nwell, ws, nullptr, out, bw, nullptr);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_well_back(const ocp_grid* g, const WellSchur& ws, const double* x, const double* bw, double* xw,
+                             cudaStream_t s) {
+  if (g->nwell == 0) return cudaSuccess;
+  const unsigned nb = well_blocks(g->nwell);
+  if (g->prm.nb == 3)
+    schur_kernel<3, false><<<nb, kWellThreads, 0, s>>>(g->d_perf, g->d_well_first, g->nwell, ws, x, nullptr, bw, xw);
+  else
+    schur_kernel<2, false><<<nb, kWellThreads, 0, s>>>(g->d_perf, g->d_well_first, g->nwell, ws, x, nullptr, bw, xw);
   return cudaGetLastError();
 }
 
@@ -281,11 +284,11 @@ ocp_status ocp_bicgstab_wells(ocp_grid* g, const double* val, const double* well
   double* bred = work + (solver_work_doubles(g) - n);
   cudaError_t e = cudaMemcpyAsync(bred, b, sizeof(double) * n, cudaMemcpyDeviceToDevice, s);
   // b' = b - B D^-1 b_w
-  if (e == cudaSuccess) e = launch_well_schur(g, ws, 1, -1.0, nullptr, bred, b_w, nullptr, s);
+  if (e == cudaSuccess) e = launch_well_reduce(g, ws, b_w, bred, s);
   if (e != cudaSuccess) return report(OCP_ERR_CUDA, "ocp_bicgstab_wells: %s", cudaGetErrorString(e));
   ocp_status st = bicgstab_run(g, val, &ws, bred, x, rtol, maxit, transpose, work, iters, relres, s);
   // x_w = D^-1 (b_w - C x), also after a solve that stopped short
-  e = launch_well_schur(g, ws, 2, 0.0, x, nullptr, b_w, x_w, s);
+  e = launch_well_back(g, ws, x, b_w, x_w, s);
   if (e != cudaSuccess) return report(OCP_ERR_CUDA, "ocp_bicgstab_wells: %s", cudaGetErrorString(e));
   return st;
 }
