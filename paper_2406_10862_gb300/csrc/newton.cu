@@ -12,51 +12,61 @@ namespace ocp {
 namespace {
 
 // Newton update with a per-cell saturation chop and the phase switch; also
-// the largest change of each variable (atomicMax on the bits of |du| >= 0,
-// which is exact and order-independent).
+// the largest change of each variable (block_max) and the number of switched
+// cells.
 template <int NB>
-__global__ void newton_update_kernel(Params P, const Table* __restrict__ gT, double* __restrict__ u,
-                                     int8_t* __restrict__ flag, const double* __restrict__ du, double scale,
-                                     double ds_max, unsigned long long* __restrict__ dmax,
-                                     int* __restrict__ nswitch) {
+__global__ void __launch_bounds__(256) newton_update_kernel(Params P, const Table* __restrict__ gT,
+                                                            double* __restrict__ u, int8_t* __restrict__ flag,
+                                                            const double* __restrict__ du, double scale,
+                                                            double ds_max, unsigned long long* __restrict__ dmax,
+                                                            int* __restrict__ nswitch) {
   const long long N = P.N;
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (c >= N) return;
-  const Table& T = *gT;
-  double d[3] = {scale * du[c * NB], scale * du[c * NB + 1], NB == 3 ? scale * du[c * NB + 2] : 0.0};
-  const int f = (NB == 3) ? flag[c] : 0;
-  // saturation chop: scale the cell's saturation changes to at most ds_max
-  double big = fabs(d[1]);
-  if (NB == 3 && f == 0) big = fmax(big, fabs(d[2]));
-  if (big > ds_max) {
-    const double sc = ds_max / big;
-    d[1] *= sc;
-    if (NB == 3 && f == 0) d[2] *= sc;
+  unsigned long long big[NB + 1] = {};
+  bool switched = false;
+  if (c < N) {
+    const Table& T = *gT;
+    double d[3] = {scale * du[c * NB], scale * du[c * NB + 1], NB == 3 ? scale * du[c * NB + 2] : 0.0};
+    const int f = (NB == 3) ? flag[c] : 0;
+    // saturation chop: scale the cell's saturation changes to at most ds_max
+    double ds = fabs(d[1]);
+    if (NB == 3 && f == 0) ds = fmax(ds, fabs(d[2]));
+    if (ds > ds_max) {
+      const double sc = ds_max / ds;
+      d[1] *= sc;
+      if (NB == 3 && f == 0) d[2] *= sc;
+    }
+    big[0] = abs_bits(d[0]);
+    big[1] = abs_bits(d[1]);
+    if (NB == 3) {
+#pragma unroll
+      for (int k = 0; k < 2; ++k) big[NB - 1 + k] = f == k ? abs_bits(d[2]) : 0ull;
+    }
+    const double p = u[c] + d[0];
+    u[c] = p;
+    u[N + c] += d[1];
+    if (NB == 3) {
+      double x = u[2 * N + c] + d[2];
+      // saturated R_s at the new pressure, from the table piece containing p
+      const int kp = segment(T.pkey, T.nrow, dkey(p));
+      const double rs_sat = fma(p - T.p[kp], T.s[4][kp], T.y[4][kp]);
+      int nf = f;
+      if (f == 0 && x < 0.0) {            // free gas disappeared: undersaturated at the bubble point
+        nf = 1;
+        x = rs_sat;
+      } else if (f == 1 && x > rs_sat) {  // more gas than the oil can hold: free gas appears
+        nf = 0;
+        x = 0.0;
+      }
+      u[2 * N + c] = x;
+      switched = nf != f;
+      if (switched) flag[c] = (int8_t)nf;
+    }
   }
-  atomicMax(&dmax[0], (unsigned long long)__double_as_longlong(fabs(d[0])));
-  atomicMax(&dmax[1], (unsigned long long)__double_as_longlong(fabs(d[1])));
-  if (NB == 3) atomicMax(&dmax[2 + f], (unsigned long long)__double_as_longlong(fabs(d[2])));
-  const double p = u[c] + d[0];
-  u[c] = p;
-  u[N + c] += d[1];
+  block_max<NB + 1>(big, dmax);
   if (NB == 3) {
-    double x = u[2 * N + c] + d[2];
-    // saturated R_s at the new pressure, from the table piece containing p
-    const int kp = segment(T.pkey, T.nrow, dkey(p));
-    const double rs_sat = fma(p - T.p[kp], T.s[4][kp], T.y[4][kp]);
-    int nf = f;
-    if (f == 0 && x < 0.0) {            // free gas disappeared: undersaturated at the bubble point
-      nf = 1;
-      x = rs_sat;
-    } else if (f == 1 && x > rs_sat) {  // more gas than the oil can hold: free gas appears
-      nf = 0;
-      x = 0.0;
-    }
-    u[2 * N + c] = x;
-    if (nf != f) {
-      flag[c] = (int8_t)nf;
-      atomicAdd(nswitch, 1);
-    }
+    const int n = __syncthreads_count(switched);
+    if (threadIdx.x == 0 && n) atomicAdd(nswitch, n);
   }
 }
 

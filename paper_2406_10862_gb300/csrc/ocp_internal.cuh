@@ -328,6 +328,37 @@ __device__ __forceinline__ void load_table(Table& T, const Table* src, unsigned 
   table_copy_wait(bar, uses, status);
 }
 
+// ------------------------------------------------------- maxima over cells
+// out[k] = max(out[k], v[k] over the CTA): the bits of non-negative doubles,
+// which order as unsigned integers (a NaN above every number), so the maxima
+// are exact whatever the order.  One atomic per CTA and value: an atomic per
+// cell on the same address serialises (a Newton update of 200 000 cells spent
+// 400 us of 418 on them).  Every thread of the CTA (a multiple of 32, at most
+// 1024) calls it.
+__device__ __forceinline__ unsigned long long abs_bits(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+}
+template <int K>
+__device__ __forceinline__ void block_max(unsigned long long (&v)[K], unsigned long long* out) {
+  __shared__ unsigned long long sm[K][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long t = __shfl_xor_sync(0xffffffffu, v[k], o);
+      v[k] = t > v[k] ? t : v[k];
+    }
+    if (lane == 0) sm[k][w] = v[k];
+  }
+  __syncthreads();
+  if (threadIdx.x < K) {
+    unsigned long long m = sm[threadIdx.x][0];
+    for (int q = 1; q < nw; ++q) m = sm[threadIdx.x][q] > m ? sm[threadIdx.x][q] : m;
+    if (m) atomicMax(out + threadIdx.x, m);
+  }
+}
+
 // ---------------------------------------------------------------- bit tricks
 // Order-preserving signed integer key of a double (total order on non-NaN).
 __host__ __device__ inline long long dkey(double x) {

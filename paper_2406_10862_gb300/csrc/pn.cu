@@ -171,37 +171,43 @@ __global__ void __launch_bounds__(128) pn_reduce_kernel(Params P, const double* 
 }
 
 template <int NB>
-__global__ void pn_update_kernel(long long N, double* __restrict__ pn, const double* __restrict__ dx, double sc,
-                                 const double* __restrict__ elim, unsigned long long* dmax) {
+__global__ void __launch_bounds__(256) pn_update_kernel(long long N, double* __restrict__ pn,
+                                                        const double* __restrict__ dx, double sc,
+                                                        const double* __restrict__ elim, unsigned long long* dmax) {
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (c >= N) return;
-  double x[NB];
-  for (int i = 0; i < NB; ++i) x[i] = dx[c * NB + i];
-  // N_w component of the full solution from the volume row
-  double xw = elim[NB * N + c];
-  for (int i = 0; i < NB; ++i) xw = fma(-elim[i * N + c], x[i], xw);
-  const double d0 = sc * x[0], dw = sc * xw;
-  pn[c] += d0;
-  pn[N + c] += dw;
-  atomicMax(&dmax[0], (unsigned long long)__double_as_longlong(fabs(d0)));
-  atomicMax(&dmax[1], (unsigned long long)__double_as_longlong(fabs(dw)));
-  for (int i = 1; i < NB; ++i) {
-    const double di = sc * x[i];
-    pn[(i + 1) * N + c] += di;
-    atomicMax(&dmax[i + 1], (unsigned long long)__double_as_longlong(fabs(di)));
+  unsigned long long big[NB + 1] = {};
+  if (c < N) {
+    double x[NB];
+    for (int i = 0; i < NB; ++i) x[i] = dx[c * NB + i];
+    // N_w component of the full solution from the volume row
+    double xw = elim[NB * N + c];
+    for (int i = 0; i < NB; ++i) xw = fma(-elim[i * N + c], x[i], xw);
+    const double d0 = sc * x[0], dw = sc * xw;
+    pn[c] += d0;
+    pn[N + c] += dw;
+    big[0] = abs_bits(d0);
+    big[1] = abs_bits(dw);
+    for (int i = 1; i < NB; ++i) {
+      const double di = sc * x[i];
+      pn[(i + 1) * N + c] += di;
+      big[i + 1] = abs_bits(di);
+    }
   }
+  block_max<NB + 1>(big, dmax);
 }
 
 template <int NB>
-__global__ void pn_norm_kernel(long long N, const double* __restrict__ phi, double scale,
-                               const double* __restrict__ res4, unsigned long long* out) {
+__global__ void __launch_bounds__(256) pn_norm_kernel(long long N, const double* __restrict__ phi, double scale,
+                                                      const double* __restrict__ res4, unsigned long long* out) {
   constexpr int L = NB + 1;
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (c >= N) return;
-  const double pv = phi[c] * scale;
-  for (int e = 0; e < NB; ++e)
-    atomicMax(&out[e], (unsigned long long)__double_as_longlong(fabs(res4[c * L + e]) / pv));
-  atomicMax(&out[3], (unsigned long long)__double_as_longlong(fabs(res4[c * L + NB])));
+  unsigned long long big[4] = {};
+  if (c < N) {
+    const double pv = phi[c] * scale;
+    for (int e = 0; e < NB; ++e) big[e] = abs_bits(fabs(res4[c * L + e]) / pv);
+    big[3] = abs_bits(res4[c * L + NB]);
+  }
+  block_max<4>(big, out);
 }
 
 // (P, N) of a natural state: N = phi S b per bulk volume (eq. 4)
