@@ -228,11 +228,15 @@ ocp_status ocp_grid_create(const ocp_grid_desc* d, int device, ocp_grid** out) {
   P.krw_max = d->krw_max; P.krg_max = d->krg_max; P.kc = d->kro_cw;
   P.pcow_max = d->pcow_max; P.pcgo_max = (nb == 3) ? d->pcgo_max : 0.0;
   P.grav_dz = 0.5 * ocp::kGrav * d->dz;
-  P.pcow2 = 2.0 * d->pcow_max;
-  P.pcgo2 = (nb == 3) ? 2.0 * d->pcgo_max : 0.0;
+  P.pcow_d = 2.0 * d->pcow_max * P.inv_w;
+  P.pcgo_d = (nb == 3) ? 2.0 * d->pcgo_max * P.inv_g : 0.0;
   P.bw_p = d->bw_ref * d->cw;
   P.rw_p = (d->bw_ref * d->cw) * d->rho_wsc;
   P.bw_p_imu = (d->bw_ref * d->cw) * P.imu_w;
+  P.krw2 = 2.0 * d->krw_max * P.inv_w;
+  P.krg2 = 2.0 * d->krg_max * P.inv_g;
+  P.inv_w2 = 2.0 * P.inv_w;
+  P.inv_og2 = 2.0 * P.inv_og;
   P.vol_rb = d->dx * d->dy * d->dz / ocp::kRbFt3;
 
   g->sms = 0;

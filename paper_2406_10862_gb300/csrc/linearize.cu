@@ -36,11 +36,27 @@ namespace ocp {
 
 namespace {
 
-// scratch layout, doubles per cell, variable-major: [field * N + cell]
+// scratch layout: tiles of 32 cells, [cell / 32][field][cell % 32], so that a
+// warp's access to a field is two whole 128-byte lines and every field of a
+// cell is at a constant offset from one address (with one array of N doubles
+// per field, each access computed a 64-bit address of its own and straddled a
+// third line).
 constexpr int kQ = 25;      // CellQ fields            0 .. 24
 constexpr int kSelf = 25;   // own residual (3) + diagonal (9)   25 .. 36
 constexpr int kPart = 37;   // after the +faces                  37 .. 48
 constexpr int kInc = 49;    // shares handed over, 3 x (F 3 + dj 9)   49 .. 84
+constexpr int kFields = 85;
+// A cell's scratch: field f is at cell_scratch(scr, c)[32 * f].
+__device__ __forceinline__ double* cell_scratch(double* scr, long long c) {
+  return scr + ((c >> 5) * (32 * kFields) + (c & 31));
+}
+// The water component's X derivative of a face flux is zero by structure
+// (neither the water's pressure, density nor mobility depends on X): it is
+// neither handed over nor added.
+template <int NB>
+__device__ __forceinline__ constexpr bool face_zero(int e, int v) {
+  return NB == 3 && e == 0 && v == 2;
+}
 
 // CellQ fields each block size reads (the two-phase path skips the gas and
 // dissolved-gas fields).
@@ -51,11 +67,11 @@ __device__ __forceinline__ bool q_used(int f) {
 }
 
 template <int NB>
-__device__ __forceinline__ void store_q(double* s, long long N, long long c, const CellQ& q) {
+__device__ __forceinline__ void store_q(double* s, const CellQ& q) {
   const double* f = reinterpret_cast<const double*>(&q);
 #pragma unroll
   for (int i = 0; i < kQ; ++i)
-    if (q_used<NB>(i)) s[i * N + c] = f[i];
+    if (q_used<NB>(i)) s[32 * i] = f[i];
 }
 // Scratch loads.  COH: the data was written earlier in the same launch by
 // another CTA (the ordered launch), so the load goes through L2, which is
@@ -66,26 +82,91 @@ __device__ __forceinline__ double lds(const double* p) {
   return *p;
 }
 template <int NB, bool COH = false>
-__device__ __forceinline__ void load_q(const double* s, long long N, long long c, CellQ& q) {
+__device__ __forceinline__ void load_q(const double* s, CellQ& q) {
   double* f = reinterpret_cast<double*>(&q);
 #pragma unroll
-  for (int i = 0; i < kQ; ++i) f[i] = q_used<NB>(i) ? lds<COH>(s + i * N + c) : 0.0;
+  for (int i = 0; i < kQ; ++i) f[i] = q_used<NB>(i) ? lds<COH>(s + 32 * i) : 0.0;
 }
 
-// Drops from L2, without writing them back to DRAM, the 128-byte lines of
-// scratch fields [f0, f1) that hold only cells [c0, c0 + TPB) (clamped to
-// N): called once every reader of those cells' scratch is done, so that dead
-// scratch costs no DRAM write.  Lines shared with other cells are left
-// alone.  All threads of the CTA call it, after a barrier.
+// Drops from L2, without writing them back to DRAM, the lines of scratch
+// fields [f0, f1) of cells [c0, c0 + TPB): called once every reader of those
+// cells' scratch is done, so that dead scratch costs no DRAM write.  A tile's
+// lines hold no other tile's cells.  All threads of the CTA call it, after a
+// barrier.
 template <int TPB>
-__device__ __forceinline__ void discard_scratch(const double* s, long long N, long long c0, int f0, int f1) {
-  constexpr int kPer = TPB / 16 >= 8 ? TPB / 8 : 8;      // power of two above the lines a range can touch
-  const long long c1 = c0 + TPB < N ? c0 + TPB : N;
-  for (int k = threadIdx.x; k < (f1 - f0) * kPer; k += blockDim.x) {
-    const int f = f0 + k / kPer, j = k % kPer;
-    const uintptr_t a = (uintptr_t)(s + f * N + c0), b = (uintptr_t)(s + f * N + c1);
-    const uintptr_t line = ((a + 127) & ~(uintptr_t)127) + 128 * (uintptr_t)j;
-    if (line + 128 <= b) asm volatile("discard.global.L2 [%0], 128;" ::"l"(line) : "memory");
+__device__ __forceinline__ void discard_scratch(double* s, long long N, long long c0, int f0, int f1) {
+  const int per = 2 * (f1 - f0);                         // 128-byte lines of 32 cells
+  for (int k = threadIdx.x; k < (TPB / 32) * per; k += blockDim.x) {
+    const long long c = c0 + 32 * (k / per);
+    if (c < N) {
+      const double* line = cell_scratch(s, c) + 32 * f0 + 16 * (k % per);
+      asm volatile("discard.global.L2 [%0], 128;" ::"l"(line) : "memory");
+    }
+  }
+}
+
+// One cell with its state loaded; SAT: its oil is saturated (as every cell's
+// of the warp).  The quantities go to scratch as soon as they are complete and
+// the rare well terms read them back, so that few values are held at a time.
+template <int NB, bool SAT>
+__device__ __forceinline__ void cell_terms(const ModelArgs& M, const Table& T, double* s, double pn, double swn,
+                                           double xn, int fn, double po, double swo, double xo, int fo, double phs,
+                                           int ip) {
+  const Params& P = M.P;
+  const int flag = SAT ? 0 : fn;
+  Pvt f;
+  pvt<NB, true>(P, T, pn, xn, flag, f);
+  {
+    Kr k;
+    CellQ q{};
+    rel_perm<NB>(P, swn, f.sg, flag, k);
+    cap_pressure<NB>(P, pn, k, q);
+    dens_mob<NB, true, true, SAT>(P, f, k, q);
+    store_q<NB>(s, q);
+  }
+  double r[3], dg[3][3];
+  if (!M.no_acc) {
+    double m[3], m_p[3], m_sw[3], m_x[3], mo[3];
+    masses<NB, true, 2, SAT>(P, f, pn, swn, phs, m, m_p, m_sw, m_x);
+    cell_masses<NB, false>(P, T, po, swo, xo, fo, phs, mo);
+    // explicitly rounded differences here and below: the terms may come
+    // from other warps (the one-cluster launch), so that no product is ever
+    // fused into these subtractions and every launch shape gives the same bits
+#pragma unroll
+    for (int e = 0; e < NB; ++e) {
+      r[e] = __dsub_rn(m[e], mo[e]);
+      dg[e][0] = m_p[e];
+      dg[e][1] = m_sw[e];
+      dg[e][2] = m_x[e];
+    }
+  } else {
+#pragma unroll
+    for (int e = 0; e < NB; ++e) r[e] = dg[e][0] = dg[e][1] = dg[e][2] = 0.0;
+  }
+  if (ip >= 0) {
+    double src[3], ds[3][3];
+    Perf w = M.perf[ip];
+    if (M.p_bh) w.p_bh = M.p_bh[w.well];
+    CellQ q;
+    load_q<NB>(s, q);
+    q.p = pn;
+    CellAux a{};
+    if (w.kind == 1) {
+      Kr k;
+      rel_perm<NB>(P, swn, f.sg, flag, k);
+      total_mob<NB>(P, f, k, true, a);
+    }
+    well_source<NB>(w, q, a, src, ds);
+    for (int e = 0; e < NB; ++e) {
+      r[e] = __dsub_rn(r[e], src[e]);
+      for (int v = 0; v < NB; ++v) dg[e][v] = __dsub_rn(dg[e][v], ds[e][v]);
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < NB; ++e) {
+    s[32 * (kSelf + e)] = r[e];
+#pragma unroll
+    for (int v = 0; v < NB; ++v) s[32 * (kSelf + 3 + 3 * e + v)] = dg[e][v];
   }
 }
 
@@ -95,7 +176,6 @@ __device__ __forceinline__ void cell_body(const ModelArgs& M, const Table& T, lo
   const long long N = P.N;
   const double* __restrict__ u_new = M.u_new;
   const double* __restrict__ u_old = M.u_old;
-  double* __restrict__ scr = M.scr;
   const double pn = u_new[c], swn = u_new[N + c], xn = (NB == 3) ? u_new[2 * N + c] : 0.0;
   const double po = u_old[c], swo = u_old[N + c], xo = (NB == 3) ? u_old[2 * N + c] : 0.0;
   const int fn = (NB == 3) ? M.f_new[c] : 0, fo = (NB == 3) ? M.f_old[c] : 0;
@@ -107,45 +187,12 @@ __device__ __forceinline__ void cell_body(const ModelArgs& M, const Table& T, lo
   // accumulation terms directly
   const double phs = M.phi[c] * M.scale;
   const int ip = M.perf_of_cell[c];
-  const bool inj = ip >= 0 && M.perf[ip].kind == 1;
-  CellQ q{};
-  CellAux a{};
-  cell_quantities<NB, true>(P, T, pn, swn, xn, fn & 1, phs, q, a, inj);
-  double r[3], dg[3][3];
-  if (!M.no_acc) {
-    double mo[3];
-    cell_masses<NB, false>(P, T, po, swo, xo, fo & 1, phs, mo);
-    // explicitly rounded differences here and below: the terms may come
-    // from other warps (the one-cluster launch), so that no product is ever
-    // fused into these subtractions and every launch shape gives the same bits
-#pragma unroll
-    for (int e = 0; e < NB; ++e) {
-      r[e] = __dsub_rn(a.m[e], mo[e]);
-      dg[e][0] = a.m_p[e];
-      dg[e][1] = a.m_sw[e];
-      dg[e][2] = a.m_x[e];
-    }
-  } else {
-#pragma unroll
-    for (int e = 0; e < NB; ++e) r[e] = dg[e][0] = dg[e][1] = dg[e][2] = 0.0;
-  }
-  if (ip >= 0) {
-    double src[3], ds[3][3];
-    Perf w = M.perf[ip];
-    if (M.p_bh) w.p_bh = M.p_bh[w.well];
-    well_source<NB>(w, q, a, src, ds);
-    for (int e = 0; e < NB; ++e) {
-      r[e] = __dsub_rn(r[e], src[e]);
-      for (int v = 0; v < NB; ++v) dg[e][v] = __dsub_rn(dg[e][v], ds[e][v]);
-    }
-  }
-  store_q<NB>(scr, N, c, q);
-#pragma unroll
-  for (int e = 0; e < NB; ++e) {
-    scr[(kSelf + e) * N + c] = r[e];
-#pragma unroll
-    for (int v = 0; v < NB; ++v) scr[(kSelf + 3 + 3 * e + v) * N + c] = dg[e][v];
-  }
+  double* s = cell_scratch(M.scr, c);
+  // warps of saturated cells leave out the terms that undersaturated oil adds
+  if (NB == 3 && !__any_sync(__activemask(), fn & 1))
+    cell_terms<NB, NB == 3>(M, T, s, pn, swn, xn, 0, po, swo, xo, fo & 1, phs, ip);
+  else
+    cell_terms<NB, false>(M, T, s, pn, swn, xn, fn & 1, po, swo, xo, fo & 1, phs, ip);
 }
 
 // The +x, +y, +z faces of cell c (BulkConn): the two off-diagonal blocks of
@@ -158,7 +205,6 @@ __device__ __forceinline__ void face_part(const ModelArgs& M, long long c, doubl
   constexpr int B2 = NB * NB;
   const Params& P = M.P;
   const long long N = P.N;
-  double* scr = M.scr;
   double* __restrict__ val = M.val;
   double* __restrict__ face_flux = M.face_flux;
   int i, j, k;
@@ -166,13 +212,14 @@ __device__ __forceinline__ void face_part(const ModelArgs& M, long long c, doubl
   const bool hm[3] = {i > 0, j > 0, k > 0};
   const bool hp[3] = {i + 1 < P.nx, j + 1 < P.ny, k + 1 < P.nz};
   const long long stride[3] = {1, P.nx, P.nxy};
+  const double* s = cell_scratch(M.scr, c);
   CellQ a;
-  load_q<NB, COH>(scr, N, c, a);
+  load_q<NB, COH>(s, a);
 #pragma unroll
   for (int e = 0; e < NB; ++e) {
-    r[e] = lds<COH>(scr + (kSelf + e) * N + c);
+    r[e] = lds<COH>(s + 32 * (kSelf + e));
 #pragma unroll
-    for (int v = 0; v < NB; ++v) dg[e][v] = lds<COH>(scr + (kSelf + 3 + 3 * e + v) * N + c);
+    for (int v = 0; v < NB; ++v) dg[e][v] = lds<COH>(s + 32 * (kSelf + 3 + 3 * e + v));
   }
   const long long row0 = row_start_ijk(P, c, i, j, k);   // the row pointers in closed form: no loads
   int slot = (int)hm[0] + (int)hm[1] + (int)hm[2] + 1;   // first + block of this row
@@ -184,8 +231,9 @@ __device__ __forceinline__ void face_part(const ModelArgs& M, long long c, doubl
       continue;
     }
     const long long n = c + stride[d];
+    double* sn = cell_scratch(M.scr, n);
     CellQ b;
-    load_q<NB, COH>(scr, N, n, b);
+    load_q<NB, COH>(sn, b);
     FaceOut<NB> o;
     const double T = M.trans[d * N + c];
     if (d == 2) face_terms<NB, true>(T, -P.grav_dz, a, b, o);
@@ -197,7 +245,7 @@ __device__ __forceinline__ void face_part(const ModelArgs& M, long long c, doubl
       r[e] += o.F[e];
 #pragma unroll
       for (int v = 0; v < NB; ++v) {
-        dg[e][v] += o.di[e][v];
+        if (!face_zero<NB>(e, v)) dg[e][v] += o.di[e][v];
         __stcs(blk + e * NB + v, o.dj[e][v]);
       }
     }
@@ -205,14 +253,14 @@ __device__ __forceinline__ void face_part(const ModelArgs& M, long long c, doubl
     // the + neighbour's row: its block of this cell, and its share
     const int slot_n = (d == 0) ? ((int)hm[2] + (int)hm[1]) : (d == 1 ? (int)hm[2] : 0);
     double* nblk = val + (row_start_ijk(P, n, i + (d == 0), j + (d == 1), k + (d == 2)) + slot_n) * B2;
-    const int base = kInc + 12 * d;
+    sn += 32 * (kInc + 12 * d);
 #pragma unroll
     for (int e = 0; e < NB; ++e) {
-      scr[(base + e) * N + n] = o.F[e];
+      sn[32 * e] = o.F[e];
 #pragma unroll
       for (int v = 0; v < NB; ++v) {
         __stcs(nblk + e * NB + v, neg(o.di[e][v]));
-        scr[(base + 3 + 3 * e + v) * N + n] = o.dj[e][v];
+        if (!face_zero<NB>(e, v)) sn[32 * (3 + 3 * e + v)] = o.dj[e][v];
       }
       if (face_flux) __stcs(face_flux + (d * NB + e) * N + c, o.F[e]);
     }
@@ -221,15 +269,14 @@ __device__ __forceinline__ void face_part(const ModelArgs& M, long long c, doubl
 
 template <int NB>
 __device__ __forceinline__ void face_body(const ModelArgs& M, long long c) {
-  const long long N = M.P.N;
-  double* scr = M.scr;
   double r[NB], dg[NB][NB];
   face_part<NB, false>(M, c, r, dg);
+  double* s = cell_scratch(M.scr, c) + 32 * kPart;
 #pragma unroll
   for (int e = 0; e < NB; ++e) {
-    scr[(kPart + e) * N + c] = r[e];
+    s[32 * e] = r[e];
 #pragma unroll
-    for (int v = 0; v < NB; ++v) scr[(kPart + 3 + 3 * e + v) * N + c] = dg[e][v];
+    for (int v = 0; v < NB; ++v) s[32 * (3 + 3 * e + v)] = dg[e][v];
   }
 }
 
@@ -240,20 +287,20 @@ template <int NB, bool COH>
 __device__ __forceinline__ void assemble_rows(const ModelArgs& M, long long c, double (&r)[NB],
                                               double (&dg)[NB][NB]) {
   const Params& P = M.P;
-  const long long N = P.N;
-  const double* scr = M.scr;
+  const double* scr = cell_scratch(M.scr, c);
   int i, j, k;
   cell_ijk(P, c, i, j, k);
   const bool hm[3] = {i > 0, j > 0, k > 0};
 #pragma unroll
   for (int d = 2; d >= 0; --d) {
     if (!hm[d]) continue;
-    const int base = kInc + 12 * d;
+    const double* s = scr + 32 * (kInc + 12 * d);
 #pragma unroll
     for (int e = 0; e < NB; ++e) {
-      r[e] -= lds<COH>(scr + (base + e) * N + c);
+      r[e] -= lds<COH>(s + 32 * e);
 #pragma unroll
-      for (int v = 0; v < NB; ++v) dg[e][v] -= lds<COH>(scr + (base + 3 + 3 * e + v) * N + c);
+      for (int v = 0; v < NB; ++v)
+        if (!face_zero<NB>(e, v)) dg[e][v] -= lds<COH>(s + 32 * (3 + 3 * e + v));
     }
   }
   double* out = M.val + (row_start_ijk(P, c, i, j, k) + (int)hm[0] + (int)hm[1] + (int)hm[2]) * NB * NB;
@@ -270,14 +317,13 @@ __device__ __forceinline__ void assemble_rows(const ModelArgs& M, long long c, d
 
 template <int NB>
 __device__ __forceinline__ void assemble_body(const ModelArgs& M, long long c) {
-  const long long N = M.P.N;
-  const double* __restrict__ scr = M.scr;
+  const double* s = cell_scratch(M.scr, c) + 32 * kPart;
   double r[NB], dg[NB][NB];
 #pragma unroll
   for (int e = 0; e < NB; ++e) {
-    r[e] = scr[(kPart + e) * N + c];
+    r[e] = s[32 * e];
 #pragma unroll
-    for (int v = 0; v < NB; ++v) dg[e][v] = scr[(kPart + 3 + 3 * e + v) * N + c];
+    for (int v = 0; v < NB; ++v) dg[e][v] = s[32 * (3 + 3 * e + v)];
   }
   assemble_rows<NB, false>(M, c, r, dg);
 }
@@ -357,7 +403,6 @@ __device__ __forceinline__ void face_dir(const ModelArgs& M, long long c, int d,
   constexpr int B2 = NB * NB;
   const Params& P = M.P;
   const long long N = P.N;
-  double* scr = M.scr;
   double* __restrict__ face_flux = M.face_flux;
   int i, j, k;
   cell_ijk(P, c, i, j, k);
@@ -370,9 +415,10 @@ __device__ __forceinline__ void face_dir(const ModelArgs& M, long long c, int d,
   }
   const long long stride = d == 0 ? 1 : (d == 1 ? (long long)P.nx : P.nxy);
   const long long n = c + stride;
+  double* sn = cell_scratch(M.scr, n);
   CellQ a, b;
-  load_q<NB, COH>(scr, N, c, a);
-  load_q<NB, COH>(scr, N, n, b);
+  load_q<NB, COH>(cell_scratch(M.scr, c), a);
+  load_q<NB, COH>(sn, b);
   FaceOut<NB> o;
   const double T = M.trans[d * N + c];
   if (d == 2) face_terms<NB, true>(T, -P.grav_dz, a, b, o);
@@ -381,17 +427,17 @@ __device__ __forceinline__ void face_dir(const ModelArgs& M, long long c, int d,
   double* blk = M.val + (row_start_ijk(P, c, i, j, k) + slot) * B2;
   const int slot_n = (d == 0) ? ((int)hm[2] + (int)hm[1]) : (d == 1 ? (int)hm[2] : 0);
   double* nblk = M.val + (row_start_ijk(P, n, i + (d == 0), j + (d == 1), k + (d == 2)) + slot_n) * B2;
-  const int base = kInc + 12 * d;
+  sn += 32 * (kInc + 12 * d);
 #pragma unroll
   for (int e = 0; e < NB; ++e) {
     own[e][lane] = o.F[e];
-    scr[(base + e) * N + n] = o.F[e];
+    sn[32 * e] = o.F[e];
 #pragma unroll
     for (int v = 0; v < NB; ++v) {
       own[3 + 3 * e + v][lane] = o.di[e][v];
       __stcs(blk + e * NB + v, o.dj[e][v]);
       __stcs(nblk + e * NB + v, neg(o.di[e][v]));
-      scr[(base + 3 + 3 * e + v) * N + n] = o.dj[e][v];
+      if (!face_zero<NB>(e, v)) sn[32 * (3 + 3 * e + v)] = o.dj[e][v];
     }
     if (face_flux) __stcs(face_flux + (d * NB + e) * N + c, o.F[e]);
   }
@@ -411,12 +457,12 @@ __device__ __forceinline__ void face_split_tile(const ModelArgs& M, long long c0
     int i, j, k;
     cell_ijk(M.P, c, i, j, k);
     const bool hp[3] = {i + 1 < M.P.nx, j + 1 < M.P.ny, k + 1 < M.P.nz};
-    double* scr = M.scr;
+    double* s = cell_scratch(M.scr, c);
     const int e = w;
-    double r = lds<COH>(scr + (kSelf + e) * N + c);
+    double r = lds<COH>(s + 32 * (kSelf + e));
     double dg[NB];
 #pragma unroll
-    for (int v = 0; v < NB; ++v) dg[v] = lds<COH>(scr + (kSelf + 3 + 3 * e + v) * N + c);
+    for (int v = 0; v < NB; ++v) dg[v] = lds<COH>(s + 32 * (kSelf + 3 + 3 * e + v));
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       if (!hp[d]) continue;
@@ -424,9 +470,9 @@ __device__ __forceinline__ void face_split_tile(const ModelArgs& M, long long c0
 #pragma unroll
       for (int v = 0; v < NB; ++v) dg[v] += own[d][3 + 3 * e + v][lane];
     }
-    scr[(kPart + e) * N + c] = r;
+    s[32 * (kPart + e)] = r;
 #pragma unroll
-    for (int v = 0; v < NB; ++v) scr[(kPart + 3 + 3 * e + v) * N + c] = dg[v];
+    for (int v = 0; v < NB; ++v) s[32 * (kPart + 3 + 3 * e + v)] = dg[v];
   }
   __syncthreads();                     // own[] is free for the next tile
 }
@@ -435,18 +481,18 @@ __device__ __forceinline__ void face_split_tile(const ModelArgs& M, long long c0
 // minus the shares of the - neighbours, in the order -z, -y, -x.
 template <int NB, bool COH>
 __device__ __forceinline__ void assemble_finish(const ModelArgs& M, long long c, int e, double r, double (&dg)[NB]) {
-  const long long N = M.P.N;
-  const double* scr = M.scr;
+  const double* scr = cell_scratch(M.scr, c);
   int i, j, k;
   cell_ijk(M.P, c, i, j, k);
   const bool hm[3] = {i > 0, j > 0, k > 0};
 #pragma unroll
   for (int d = 2; d >= 0; --d) {
     if (!hm[d]) continue;
-    const int base = kInc + 12 * d;
-    r -= lds<COH>(scr + (base + e) * N + c);
+    const double* s = scr + 32 * (kInc + 12 * d);
+    r -= lds<COH>(s + 32 * e);
 #pragma unroll
-    for (int v = 0; v < NB; ++v) dg[v] -= lds<COH>(scr + (base + 3 + 3 * e + v) * N + c);
+    for (int v = 0; v < NB; ++v)
+      if (!face_zero<NB>(e, v)) dg[v] -= lds<COH>(s + 32 * (3 + 3 * e + v));
   }
   double* out = M.val + (row_start_ijk(M.P, c, i, j, k) + (int)hm[0] + (int)hm[1] + (int)hm[2]) * NB * NB;
   __stcs(M.res + c * NB + e, r);
@@ -457,12 +503,11 @@ __device__ __forceinline__ void assemble_finish(const ModelArgs& M, long long c,
 
 template <int NB, bool COH>
 __device__ __forceinline__ void assemble_split_row(const ModelArgs& M, long long c, int e) {
-  const long long N = M.P.N;
-  const double* scr = M.scr;
-  const double r = lds<COH>(scr + (kPart + e) * N + c);
+  const double* s = cell_scratch(M.scr, c) + 32 * kPart;
+  const double r = lds<COH>(s + 32 * e);
   double dg[NB];
 #pragma unroll
-  for (int v = 0; v < NB; ++v) dg[v] = lds<COH>(scr + (kPart + 3 + 3 * e + v) * N + c);
+  for (int v = 0; v < NB; ++v) dg[v] = lds<COH>(s + 32 * (3 + 3 * e + v));
   assemble_finish<NB, COH>(M, c, e, r, dg);
 }
 
@@ -945,7 +990,8 @@ __device__ __forceinline__ void cluster_face_stage(const ModelArgs& M, long long
         di_o[v] = B.oil[d][1 + v][lane];
         dj_o[v] = B.oil[d][4 + v][lane];
       }
-      gas_component(a, b, B.up_o[d][lane] != 0, Fo, di_o, dj_o, Fp, di, dj, F, dig, djg);
+      if (d == 2) gas_component<true>(a, b, B.up_o[d][lane] != 0, Fo, di_o, dj_o, Fp, di, dj, F, dig, djg);
+      else gas_component<false>(a, b, B.up_o[d][lane] != 0, Fo, di_o, dj_o, Fp, di, dj, F, dig, djg);
       face_row<NB>(M, c, d, 2, blk, nblk, F, dig, djg, B.own[d], lane, sh);
     }
   }
@@ -1435,8 +1481,12 @@ cudaError_t preload_linearize(int nb) {
   return e;
 }
 
-// 85 doubles per cell are used; 100 are reserved.
-int64_t linearize_scratch_doubles(int64_t N) { return (int64_t)100 * N; }
+// kFields doubles per cell, in whole tiles of 32 cells; 100 per cell are
+// reserved (the IMPEC path keeps its own layout in them).
+int64_t linearize_scratch_doubles(int64_t N) {
+  const int64_t tiles = (N + 31) / 32 * 32 * kFields;
+  return tiles > 100 * N ? tiles : 100 * N;
+}
 
 cudaError_t launch_linearize(const ocp_grid* g, const double* u_new, const int8_t* f_new,
                              const double* u_old, const int8_t* f_old, double dt, double* res,

@@ -57,9 +57,11 @@ struct Params {
   double vol_rb;                          // cell bulk volume in rb
   unsigned long long nx_m, ny_m;          // exact division by nx and ny: q = (c * m) >> (32 + s)
   int nx_s, ny_s;
-  double pcow2, pcgo2;                    // 2 Pc_max (derivative factors)
+  double pcow_d, pcgo_d;                  // 2 Pc_max times the slope of the normalised saturation
   double bw_p;                            // d b_w / dp
   double rw_p, bw_p_imu;                  // d rho_w / dp, (d b_w / dp) / mu_w
+  double krw2, krg2;                      // 2 kr_max times the slope of the normalised saturation
+  double inv_w2, inv_og2;                 // 2 inv_w, 2 inv_og
 };
 
 // Well perforation data on the device (one entry per perforated cell).
@@ -228,18 +230,19 @@ __device__ __forceinline__ void cell_ijk(const Params& P, long long c, int& i, i
 }
 // Number of stored blocks in the rows before cell c = (i, j, k): 7 per
 // earlier cell minus the missing neighbours of every earlier cell, in
-// closed form.
+// closed form.  Block indices fit 32 bits (ocp_grid_create rejects 7 N >=
+// 2^31), where an add is one instruction instead of two.
 __device__ __forceinline__ long long row_start_ijk(const Params& P, long long c, int i, int j, int k) {
-  const long long nx = P.nx, nxy = P.nxy, N = P.N;
-  const long long q = (long long)k * P.ny + j;            // c / nx
-  const long long i0 = q + (i > 0);                        // earlier cells with i == 0
-  const long long iL = q;                                  // ... with i == nx-1
-  const long long rem = (long long)j * nx + i;             // c % nxy
-  const long long j0 = k * nx + (rem < nx ? rem : nx);     // ... with j == 0
-  const long long jL = k * nx + (rem > nxy - nx ? rem - (nxy - nx) : 0);
-  const long long k0 = c < nxy ? c : nxy;                  // ... with k == 0
-  const long long kL = c > N - nxy ? c - (N - nxy) : 0;    // ... with k == nz-1
-  return 7 * c - (i0 + iL + j0 + jL + k0 + kL);
+  const int nx = P.nx, nxy = (int)P.nxy, N = (int)P.N, ci = (int)c;
+  const int q = k * P.ny + j;                    // c / nx
+  const int i0 = q + (i > 0);                    // earlier cells with i == 0
+  const int iL = q;                              // ... with i == nx-1
+  const int rem = j * nx + i;                    // c % nxy
+  const int j0 = k * nx + min(rem, nx);          // ... with j == 0
+  const int jL = k * nx + max(rem - (nxy - nx), 0);
+  const int k0 = min(ci, nxy);                   // ... with k == 0
+  const int kL = max(ci - (N - nxy), 0);         // ... with k == nz-1
+  return (long long)(7 * ci - (i0 + iL + j0 + jL + k0 + kL));
 }
 
 // ------------------------------------------------- programmatic launches
@@ -378,6 +381,10 @@ __device__ __forceinline__ bool finite(double x) {
   return ((__double2hiint(x) >> 20) & 0x7ff) != 0x7ff;
 }
 __device__ __forceinline__ double sel(bool c, double a, double b) { return c ? a : b; }
+// x != 0 (or NaN), without an FP64 compare.
+__device__ __forceinline__ bool nonzero(double x) {
+  return ((unsigned)__double2loint(x) | ((unsigned)__double2hiint(x) & 0x7fffffffu)) != 0u;
+}
 
 // Largest k <= nrow-2 with key[k] <= xk (binary search on integer keys).
 __device__ __forceinline__ int segment(const long long* key, int nrow, long long xk) {
@@ -389,17 +396,19 @@ __device__ __forceinline__ int segment(const long long* key, int nrow, long long
   return lo;
 }
 
-// Power with a constant exponent >= 1 and its derivative; exponent 2 uses a
-// product.  s is already clamped to [0, 1].
-__device__ __forceinline__ void cpow(double s, double n, int sq, double& v, double& d) {
-  if (sq) { v = s * s; d = s + s; }
-  else { v = pow(s, n); d = n * pow(s, n - 1.0); }
+// Power with a constant exponent >= 1 and its derivative times the slope ds
+// of s, as a product of the two values (d, ds2); exponent 2 uses products,
+// with the factor 2 taken into the slope.  s is already clamped to [0, 1].
+__device__ __forceinline__ void cpow(double s, double n, int sq, double ds, double ds2, double& v, double& d,
+                                     double& slope) {
+  if (sq) { v = s * s; d = s; slope = ds2; }
+  else { v = pow(s, n); d = n * pow(s, n - 1.0); slope = ds; }
 }
 
-// Clamp a normalised saturation to [0, 1]: outside, value clamped and slope 0.
-__device__ __forceinline__ void clamp01(double& s, double& ds) {
-  if (!nonneg(s)) { s = 0.0; ds = 0.0; }
-  else if (dkey(s) > dkey(1.0)) { s = 1.0; ds = 0.0; }
+// Clamp a normalised saturation to [0, 1]: outside, value clamped and slopes 0.
+__device__ __forceinline__ void clamp01(double& s, double& ds, double& ds2) {
+  if (!nonneg(s)) { s = 0.0; ds = ds2 = 0.0; }
+  else if (dkey(s) > dkey(1.0)) { s = 1.0; ds = ds2 = 0.0; }
 }
 
 // ------------------------------------------------------------ cell quantities
@@ -496,8 +505,10 @@ __device__ __forceinline__ void pvt(const Params& P, const Table& T, double p, d
 // with DERIV their derivatives with respect to (p, S_w, X).  Used for both
 // time levels, so that an unchanged state gives an exactly zero accumulation.
 // PART 2 computes every component, PART 0 only water and oil, PART 1 only
-// gas (so that the components can be split between warps).
-template <int NB, bool DERIV, int PART = 2>
+// gas (so that the components can be split between warps).  SAT: the caller
+// knows the oil to be saturated (b_o and R_s do not depend on X = S_g); the
+// terms that are zero then are left out, the others are the same bits.
+template <int NB, bool DERIV, int PART = 2, bool SAT = false>
 __device__ __forceinline__ void masses(const Params& P, const Pvt& f, double p, double sw, double phi_ref,
                                        double* m, double* m_p, double* m_sw, double* m_x) {
   const double phi = phi_ref * fma(P.cr, p - P.p_ref, 1.0);
@@ -517,12 +528,13 @@ __device__ __forceinline__ void masses(const Params& P, const Pvt& f, double p, 
       m_x[0] = 0.0;
       m_p[1] = fma(phi_p, sob, phi * so * f.bo_p);
       m_sw[1] = -phi * f.bo;
-      m_x[1] = phi * fma(so_x, f.bo, so * f.bo_x);
+      m_x[1] = SAT ? m_sw[1] : phi * fma(so_x, f.bo, so * f.bo_x);
     }
     if (PART != 0 && NB == 3) {
       const double G = fma(f.sg, f.bg, f.rs * sob);
       const double G_p = fma(f.sg, f.bg_p, fma(f.rs_p, sob, f.rs * so * f.bo_p));
-      const double G_x = fma(f.sg_x, f.bg, fma(f.rs_x, sob, f.rs * fma(so_x, f.bo, so * f.bo_x)));
+      const double G_x = SAT ? __dadd_rn(f.bg, -__dmul_rn(f.rs, f.bo))
+                             : fma(f.sg_x, f.bg, fma(f.rs_x, sob, f.rs * fma(so_x, f.bo, so * f.bo_x)));
       m_p[2] = fma(phi_p, G, phi * G_p);
       m_sw[2] = -phi * f.rs * f.bo;
       m_x[2] = phi * G_x;
@@ -545,41 +557,46 @@ struct Kr {
 // combines them (so that the two sides can also run in different warps).
 struct KrSide {
   double s, s_d;               // clamped normalised S_w or S_g and its slope
-  double so_d;                 // slope of the normalised oil saturation of the curve
-  double po, dpo;              // (s_ow or s_og)^n and its derivative
+  double po, dpo, so_d;        // (s_ow or s_og)^n; its derivative in S_w or S_g is dpo so_d
   double kr, kr_d;             // k_rw or k_rg and its derivative in S_w or S_g
 };
+// kr_d = kr_max (d s^n) (slope) in one product for exponent 2: the constants
+// kr_max * 2 slope are precomputed.
 __device__ __forceinline__ void rel_perm_w(const Params& P, double sw, KrSide& w) {
-  double s_w = (sw - P.swc) * P.inv_w, s_w_d = P.inv_w;
-  clamp01(s_w, s_w_d);
-  double s_ow = (1.0 - sw - P.sorw) * P.inv_w, s_ow_d = -P.inv_w;
-  clamp01(s_ow, s_ow_d);
-  double pw_, dw_, pow_, dow_;
-  cpow(s_w, P.nw, P.sq_w, pw_, dw_);
-  cpow(s_ow, P.now, P.sq_ow, pow_, dow_);
+  double s_w = (sw - P.swc) * P.inv_w, s_w_d = P.inv_w, s_w_k = P.krw2;
+  clamp01(s_w, s_w_d, s_w_k);
+  double s_ow = (1.0 - sw - P.sorw) * P.inv_w, s_ow_d = -P.inv_w, s_ow_2 = -P.inv_w2;
+  clamp01(s_ow, s_ow_d, s_ow_2);
+  double pw_;
+  if (P.sq_w) {
+    pw_ = s_w * s_w;
+    w.kr_d = s_w_k * s_w;
+  } else {
+    pw_ = pow(s_w, P.nw);
+    w.kr_d = P.krw_max * (P.nw * pow(s_w, P.nw - 1.0)) * s_w_d;
+  }
+  cpow(s_ow, P.now, P.sq_ow, s_ow_d, s_ow_2, w.po, w.dpo, w.so_d);
   w.s = s_w;
   w.s_d = s_w_d;
-  w.so_d = s_ow_d;
-  w.po = pow_;
-  w.dpo = dow_;
   w.kr = P.krw_max * pw_;
-  w.kr_d = P.krw_max * dw_ * s_w_d;
 }
 __device__ __forceinline__ void rel_perm_g(const Params& P, double sg, KrSide& g) {
-  double s_g = (sg - P.sgc) * P.inv_g, s_g_d = P.inv_g;
-  clamp01(s_g, s_g_d);
-  double s_og = (1.0 - sg - P.swc - P.sorg) * P.inv_og, s_og_d = -P.inv_og;
-  clamp01(s_og, s_og_d);
-  double pg_, dg_, pog_, dog_;
-  cpow(s_g, P.ng, P.sq_g, pg_, dg_);
-  cpow(s_og, P.nog, P.sq_og, pog_, dog_);
+  double s_g = (sg - P.sgc) * P.inv_g, s_g_d = P.inv_g, s_g_k = P.krg2;
+  clamp01(s_g, s_g_d, s_g_k);
+  double s_og = (1.0 - sg - P.swc - P.sorg) * P.inv_og, s_og_d = -P.inv_og, s_og_2 = -P.inv_og2;
+  clamp01(s_og, s_og_d, s_og_2);
+  double pg_;
+  if (P.sq_g) {
+    pg_ = s_g * s_g;
+    g.kr_d = s_g_k * s_g;
+  } else {
+    pg_ = pow(s_g, P.ng);
+    g.kr_d = P.krg_max * (P.ng * pow(s_g, P.ng - 1.0)) * s_g_d;
+  }
+  cpow(s_og, P.nog, P.sq_og, s_og_d, s_og_2, g.po, g.dpo, g.so_d);
   g.s = s_g;
   g.s_d = s_g_d;
-  g.so_d = s_og_d;
-  g.po = pog_;
-  g.dpo = dog_;
   g.kr = P.krg_max * pg_;
-  g.kr_d = P.krg_max * dg_ * s_g_d;
 }
 // k_ro (Stone II with three phases, the oil-water curve with two) from the
 // two sides; the sums are explicitly rounded so that they never take in a
@@ -635,16 +652,16 @@ __device__ __forceinline__ void cap_pressure(const Params& P, double p, const Kr
   const double omw = 1.0 - k.s_w;
   q.p = p;
   q.pw = p - P.pcow_max * (omw * omw);
-  q.dpw_sw = P.pcow2 * omw * k.s_w_d;
+  q.dpw_sw = nonzero(k.s_w_d) ? P.pcow_d * omw : 0.0;
   if (NB == 3) {
     q.pg = p + P.pcgo_max * (k.s_g * k.s_g);
-    q.dpg_x = k.gx ? P.pcgo2 * k.s_g * k.s_g_d : 0.0;
+    q.dpg_x = k.gx && nonzero(k.s_g_d) ? P.pcgo_d * k.s_g : 0.0;
   }
 }
 
 // Phase densities and mobilities lambda = k_r b / mu with their derivatives:
-// water and gas (WG), oil (O), or all.
-template <int NB, bool WG = true, bool O = true>
+// water and gas (WG), oil (O), or all.  SAT as for masses.
+template <int NB, bool WG = true, bool O = true, bool SAT = false>
 __device__ __forceinline__ void dens_mob(const Params& P, const Pvt& f, const Kr& k, CellQ& q) {
   if (WG) {
     q.rw = f.bw * P.rho_wsc;
@@ -669,14 +686,19 @@ __device__ __forceinline__ void dens_mob(const Params& P, const Pvt& f, const Kr
   const double ro0 = fma(f.rs, P.cg, P.rho_osc);
   q.ro = ro0 * f.bo;
   q.ro_p = fma(P.cg * f.rs_p, f.bo, ro0 * f.bo_p);
-  q.ro_x = fma(P.cg * f.rs_x, f.bo, ro0 * f.bo_x);
   const double bmo = f.bo * f.imo;
   const double bmo_p = fma(f.bo_p, f.imo, f.bo * f.imo_p);
-  const double bmo_x = fma(f.bo_x, f.imo, f.bo * f.imo_x);
   q.lo = k.kro * bmo;
   q.lo_p = k.kro * bmo_p;
   q.lo_sw = k.kro_sw * bmo;
-  q.lo_x = fma(k.kro_x, bmo, k.kro * bmo_x);
+  if (SAT) {
+    q.ro_x = 0.0;
+    q.lo_x = k.kro_x * bmo;
+  } else {
+    q.ro_x = fma(P.cg * f.rs_x, f.bo, ro0 * f.bo_x);
+    const double bmo_x = fma(f.bo_x, f.imo, f.bo * f.imo_x);
+    q.lo_x = fma(k.kro_x, bmo, k.kro * bmo_x);
+  }
 }
 
 // Total mobility sum k_r / mu and the injected phases' b (injector cells;
@@ -749,6 +771,10 @@ __device__ __forceinline__ double neg(double x) {
 //   PX   the phase pressure depends on X (gas, through Pc_go), d = dpa;
 //   RX   the density depends on X (oil, through R_s);
 //   LSW, LX  the mobility depends on S_w, X.
+//
+// Only the upstream cell's mobility enters, so its derivatives are added on
+// that side alone: without gravity d F / d p is -+T lambda_up on the
+// downstream side and takes one FMA on the upstream side.
 template <bool GRAV, bool PSW, bool PX, bool RX, bool LSW, bool LX>
 __device__ __forceinline__ void phase_flux(double T, double hz, double pa_i, double pa_j, double dpa_i,
                                            double dpa_j, double rho_i, double rho_j, double rho_p_i,
@@ -762,13 +788,15 @@ __device__ __forceinline__ void phase_flux(double T, double hz, double pa_i, dou
   const double Tl = T * sel(up, l_i, l_j);
   const double Td = T * dphi;
   F = Tl * dphi;
-  const double ulp = Td * sel(up, l_p_i, l_p_j);
+  const double lp = sel(up, l_p_i, l_p_j);
   if (GRAV) {
+    const double ulp = Td * lp;
     di[0] = fma(Tl, fma(-rho_p_i, hz, 1.0), sel(up, ulp, 0.0));
     dj[0] = fma(Tl, fma(-rho_p_j, hz, -1.0), sel(up, 0.0, ulp));
   } else {
-    di[0] = Tl + sel(up, ulp, 0.0);
-    dj[0] = sel(up, 0.0, ulp) - Tl;
+    const double U = fma(Td, lp, sel(up, Tl, neg(Tl)));
+    di[0] = sel(up, U, Tl);
+    dj[0] = sel(up, neg(Tl), U);
   }
   double usw = 0.0;
   if (LSW) usw = Td * sel(up, l_sw_i, l_sw_j);
@@ -781,21 +809,18 @@ __device__ __forceinline__ void phase_flux(double T, double hz, double pa_i, dou
   }
   double ux = 0.0;
   if (LX) ux = Td * sel(up, l_x_i, l_x_j);
-  constexpr bool CX = PX || (GRAV && RX);   // dphi depends on X
-  if (CX) {
-    double cx_i, cx_j;
-    if (PX) {
-      cx_i = dpa_i;
-      cx_j = neg(dpa_j);
-    } else {
-      cx_i = neg(rho_x_i * hz);
-      cx_j = neg(rho_x_j * hz);
+  di[2] = sel(up, ux, 0.0);
+  dj[2] = sel(up, 0.0, ux);
+  if (PX) {
+    di[2] = fma(Tl, dpa_i, di[2]);
+    dj[2] = fma(Tl, neg(dpa_j), dj[2]);
+  } else if (GRAV && RX) {
+    // saturated oil: the densities do not depend on X, and adding the zero
+    // products changes nothing (where that holds for the whole warp)
+    if (__any_sync(__activemask(), nonzero(rho_x_i) || nonzero(rho_x_j))) {
+      di[2] = fma(Tl, neg(rho_x_i * hz), di[2]);
+      dj[2] = fma(Tl, neg(rho_x_j * hz), dj[2]);
     }
-    di[2] = fma(Tl, cx_i, sel(up, ux, 0.0));
-    dj[2] = fma(Tl, cx_j, sel(up, 0.0, ux));
-  } else {
-    di[2] = sel(up, ux, 0.0);
-    dj[2] = sel(up, 0.0, ux);
   }
 }
 
@@ -837,21 +862,30 @@ __device__ __forceinline__ void gas_flux(double T, double hz, const CellQ& a, co
                                                      a.lg_x, b.lg_x, F, di, dj, up);
 }
 // The gas component: free gas plus the gas dissolved in the upstream oil
-// (Fo, di_o, dj_o, up_o the oil phase; Fg, dg_i, dg_j the gas phase).
+// (Fo, di_o, dj_o, up_o the oil phase; Fg, dg_i, dg_j the gas phase).  On the
+// oil's downstream side its flux depends on p, with gravity on X too, and
+// never on S_w.
+template <bool GRAV>
 __device__ __forceinline__ void gas_component(const CellQ& a, const CellQ& b, bool up_o, double Fo,
                                               const double (&di_o)[3], const double (&dj_o)[3], double Fg,
                                               const double (&dg_i)[3], const double (&dg_j)[3], double& F,
                                               double (&di)[3], double (&dj)[3]) {
   const double rsu = sel(up_o, a.rs, b.rs);
   F = fma(rsu, Fo, Fg);
-  const double frp = Fo * sel(up_o, a.rs_p, b.rs_p);
-  const double frx = Fo * sel(up_o, a.rs_x, b.rs_x);
-  di[0] = fma(rsu, di_o[0], dg_i[0]) + sel(up_o, frp, 0.0);
-  dj[0] = fma(rsu, dj_o[0], dg_j[0]) + sel(up_o, 0.0, frp);
-  di[1] = rsu * di_o[1];
-  dj[1] = rsu * dj_o[1];
-  di[2] = fma(rsu, di_o[2], dg_i[2]) + sel(up_o, frx, 0.0);
-  dj[2] = fma(rsu, dj_o[2], dg_j[2]) + sel(up_o, 0.0, frx);
+  const double U0 = fma(sel(up_o, a.rs_p, b.rs_p), Fo,
+                        fma(rsu, sel(up_o, di_o[0], dj_o[0]), sel(up_o, dg_i[0], dg_j[0])));
+  const double D0 = fma(rsu, sel(up_o, dj_o[0], di_o[0]), sel(up_o, dg_j[0], dg_i[0]));
+  const double U1 = rsu * sel(up_o, di_o[1], dj_o[1]);
+  const double U2 = fma(sel(up_o, a.rs_x, b.rs_x), Fo,
+                        fma(rsu, sel(up_o, di_o[2], dj_o[2]), sel(up_o, dg_i[2], dg_j[2])));
+  double D2 = sel(up_o, dg_j[2], dg_i[2]);
+  if (GRAV) D2 = fma(rsu, sel(up_o, dj_o[2], di_o[2]), D2);
+  di[0] = sel(up_o, U0, D0);
+  dj[0] = sel(up_o, D0, U0);
+  di[1] = sel(up_o, U1, 0.0);
+  dj[1] = sel(up_o, 0.0, U1);
+  di[2] = sel(up_o, U2, D2);
+  dj[2] = sel(up_o, D2, U2);
 }
 
 template <int NB, bool GRAV>
@@ -861,10 +895,15 @@ __device__ __forceinline__ void face_terms(double T, double hz, const CellQ& a, 
   water_flux<NB, GRAV>(T, hz, a, b, o.F[0], o.di[0], o.dj[0], up_w);
   oil_flux<NB, GRAV>(T, hz, a, b, o.F[1], o.di[1], o.dj[1], up_o);
   if (NB == 3) {
-    double Fg, dg_i[3], dg_j[3];
-    bool up_g;
-    gas_flux<NB, GRAV>(T, hz, a, b, Fg, dg_i, dg_j, up_g);
-    gas_component(a, b, up_o, o.F[1], o.di[1], o.dj[1], Fg, dg_i, dg_j, o.F[NB - 1], o.di[NB - 1],
+    double Fg = 0.0, dg_i[3] = {0.0, 0.0, 0.0}, dg_j[3] = {0.0, 0.0, 0.0};
+    // no free gas in the warp's cells: the phase's flux and derivatives are zero
+    const bool gas = nonzero(a.lg) || nonzero(a.lg_p) || nonzero(a.lg_x) || nonzero(b.lg) || nonzero(b.lg_p) ||
+                     nonzero(b.lg_x);
+    if (__any_sync(__activemask(), gas)) {
+      bool up_g;
+      gas_flux<NB, GRAV>(T, hz, a, b, Fg, dg_i, dg_j, up_g);
+    }
+    gas_component<GRAV>(a, b, up_o, o.F[1], o.di[1], o.dj[1], Fg, dg_i, dg_j, o.F[NB - 1], o.di[NB - 1],
                   o.dj[NB - 1]);
   }
 }
