@@ -274,11 +274,9 @@ ocp_status ocp_batch_get_status(ocp_batch* batch, void* cuda_stream);
 
 /* Launch shape of ocp_linearize on one grid (for example one found by
  * ocp_batch_tune on a batch of that grid alone).  A new grid starts with one
- * CTA per tile and the largest tiles (128 cells for the cell and face stages,
- * 256 for assembly) that still give every SM two CTAs, halving down to 32
- * cells for small grids; grids of fewer than 64 cells per SM start with
- * ordered = 3, and grids that fit one cluster (ocp_grid_cluster_tiles) with
- * ordered = 4. */
+ * CTA per tile, tiles of 64 cells for the cell stage and 32 for the face and
+ * assembly stages; grids of fewer than 128 cells per SM start with ordered = 3,
+ * and grids that fit one cluster (ocp_grid_cluster_tiles) with ordered = 4. */
 ocp_status ocp_grid_set_shape(ocp_grid* grid, const ocp_launch_shape* shape);
 /* The launch shape ocp_linearize currently uses on the grid. */
 ocp_status ocp_grid_get_shape(const ocp_grid* grid, ocp_launch_shape* shape);

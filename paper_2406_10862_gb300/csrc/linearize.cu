@@ -195,13 +195,62 @@ __device__ __forceinline__ void cell_body(const ModelArgs& M, const Table& T, lo
     cell_terms<NB, false>(M, T, s, pn, swn, xn, fn & 1, po, swo, xo, fo & 1, phs, ip);
 }
 
+// ------------------------------------------------------------ block stores
+// A warp's blocks go to the Jacobian through shared memory.  Each lane's 3x3
+// block is 72 contiguous bytes, but its neighbour lane's lies a whole row
+// (about 500 bytes) away, so one store per lane and entry touches 32 lines and
+// writes 8 bytes of each: at 200 000 cells 65 sectors a cell went through the
+// L1's store path, the loads behind them waited, and the face stage's warps
+// spent 36 % of their time on that.  Storing the 288 values in block order
+// instead, nine lanes to a block, touches four lines at a time.  A 2x2 block
+// is one 32-byte sector: a single wide store where the matrix is aligned to it.
+template <int NB>
+struct WarpStage {
+  double v[NB == 3 ? 32 * 9 : 1];
+  double* p[NB == 3 ? 32 : 1];
+};
+// Stores block b of every lane of the warp at its base (null: none).
+template <int NB>
+__device__ __forceinline__ void store_blocks(WarpStage<NB>& st, const double (&b)[NB][NB], double* base) {
+  if constexpr (NB == 3) {
+    const int lane = threadIdx.x & 31;
+    if (base) {
+#pragma unroll
+      for (int e = 0; e < 3; ++e)
+#pragma unroll
+        for (int v = 0; v < 3; ++v) st.v[9 * lane + 3 * e + v] = b[e][v];
+    }
+    st.p[lane] = base;
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      const int q = 32 * k + lane, r = (q * 57) >> 9;    // q / 9 for q < 288
+      double* p = st.p[r];
+      if (p) __stcs(p + (q - 9 * r), st.v[q]);
+    }
+    __syncwarp();
+  } else if (base) {
+    if (((uintptr_t)base & 31) == 0) {
+      asm volatile("st.global.cs.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(base), "d"(b[0][0]), "d"(b[0][1]), "d"(b[1][0]),
+                   "d"(b[1][1])
+                   : "memory");
+    } else {
+#pragma unroll
+      for (int e = 0; e < NB; ++e)
+#pragma unroll
+        for (int v = 0; v < NB; ++v) __stcs(base + e * NB + v, b[e][v]);
+    }
+  }
+}
+
 // The +x, +y, +z faces of cell c (BulkConn): the two off-diagonal blocks of
 // each face go straight into the Jacobian, the + neighbour's share (flux and
 // diagonal block) into its scratch slots, and this row's residual and
 // diagonal block -- its own terms plus its + faces -- come back in r, dg.
+// Whole warps call it; `live` is false past the last cell.
 template <int NB, bool COH>
-__device__ __forceinline__ void face_part(const ModelArgs& M, long long c, double (&r)[NB],
-                                          double (&dg)[NB][NB]) {
+__device__ __forceinline__ void face_part(const ModelArgs& M, long long c, bool live, WarpStage<NB>& st,
+                                          double (&r)[NB], double (&dg)[NB][NB]) {
   constexpr int B2 = NB * NB;
   const Params& P = M.P;
   const long long N = P.N;
@@ -210,67 +259,72 @@ __device__ __forceinline__ void face_part(const ModelArgs& M, long long c, doubl
   int i, j, k;
   cell_ijk(P, c, i, j, k);
   const bool hm[3] = {i > 0, j > 0, k > 0};
-  const bool hp[3] = {i + 1 < P.nx, j + 1 < P.ny, k + 1 < P.nz};
+  const bool hp[3] = {live && i + 1 < P.nx, live && j + 1 < P.ny, live && k + 1 < P.nz};
   const long long stride[3] = {1, P.nx, P.nxy};
   const double* s = cell_scratch(M.scr, c);
   CellQ a;
-  load_q<NB, COH>(s, a);
+  if (live) {
+    load_q<NB, COH>(s, a);
 #pragma unroll
-  for (int e = 0; e < NB; ++e) {
-    r[e] = lds<COH>(s + 32 * (kSelf + e));
+    for (int e = 0; e < NB; ++e) {
+      r[e] = lds<COH>(s + 32 * (kSelf + e));
 #pragma unroll
-    for (int v = 0; v < NB; ++v) dg[e][v] = lds<COH>(s + 32 * (kSelf + 3 + 3 * e + v));
+      for (int v = 0; v < NB; ++v) dg[e][v] = lds<COH>(s + 32 * (kSelf + 3 + 3 * e + v));
+    }
   }
   const long long row0 = row_start_ijk(P, c, i, j, k);   // the row pointers in closed form: no loads
   int slot = (int)hm[0] + (int)hm[1] + (int)hm[2] + 1;   // first + block of this row
 #pragma unroll 1
   for (int d = 0; d < 3; ++d) {
-    if (!hp[d]) {
-      if (face_flux)
-        for (int e = 0; e < NB; ++e) face_flux[(d * NB + e) * N + c] = 0.0;
-      continue;
-    }
-    const long long n = c + stride[d];
-    double* sn = cell_scratch(M.scr, n);
-    CellQ b;
-    load_q<NB, COH>(sn, b);
     FaceOut<NB> o;
-    const double T = M.trans[d * N + c];
-    if (d == 2) face_terms<NB, true>(T, -P.grav_dz, a, b, o);
-    else face_terms<NB, false>(T, 0.0, a, b, o);
-    // this row: flux out, diagonal, and the block of the + neighbour
-    double* blk = val + (row0 + slot) * B2;
+    double blk[NB][NB], *base = nullptr, *nbase = nullptr;
+    if (hp[d]) {
+      const long long n = c + stride[d];
+      double* sn = cell_scratch(M.scr, n);
+      CellQ b;
+      load_q<NB, COH>(sn, b);
+      const double T = M.trans[d * N + c];
+      if (d == 2) face_terms<NB, true>(T, -P.grav_dz, a, b, o);
+      else face_terms<NB, false>(T, 0.0, a, b, o);
+      // this row: flux out, diagonal, and the block of the + neighbour; the
+      // + neighbour's row: its share, and its block of this cell
+      base = val + (row0 + slot) * B2;
+      ++slot;
+      const int slot_n = (d == 0) ? ((int)hm[2] + (int)hm[1]) : (d == 1 ? (int)hm[2] : 0);
+      nbase = val + (row_start_ijk(P, n, i + (d == 0), j + (d == 1), k + (d == 2)) + slot_n) * B2;
+      sn += 32 * (kInc + 12 * d);
 #pragma unroll
-    for (int e = 0; e < NB; ++e) {
-      r[e] += o.F[e];
+      for (int e = 0; e < NB; ++e) {
+        r[e] += o.F[e];
+        sn[32 * e] = o.F[e];
 #pragma unroll
-      for (int v = 0; v < NB; ++v) {
-        if (!face_zero<NB>(e, v)) dg[e][v] += o.di[e][v];
-        __stcs(blk + e * NB + v, o.dj[e][v]);
+        for (int v = 0; v < NB; ++v) {
+          blk[e][v] = o.dj[e][v];
+          if (!face_zero<NB>(e, v)) {
+            dg[e][v] += o.di[e][v];
+            sn[32 * (3 + 3 * e + v)] = o.dj[e][v];
+          }
+        }
+        if (face_flux) __stcs(face_flux + (d * NB + e) * N + c, o.F[e]);
       }
+    } else if (live && face_flux) {
+      for (int e = 0; e < NB; ++e) face_flux[(d * NB + e) * N + c] = 0.0;
     }
-    ++slot;
-    // the + neighbour's row: its block of this cell, and its share
-    const int slot_n = (d == 0) ? ((int)hm[2] + (int)hm[1]) : (d == 1 ? (int)hm[2] : 0);
-    double* nblk = val + (row_start_ijk(P, n, i + (d == 0), j + (d == 1), k + (d == 2)) + slot_n) * B2;
-    sn += 32 * (kInc + 12 * d);
+    if (!__any_sync(0xffffffffu, hp[d])) continue;
+    store_blocks<NB>(st, blk, base);
 #pragma unroll
-    for (int e = 0; e < NB; ++e) {
-      sn[32 * e] = o.F[e];
+    for (int e = 0; e < NB; ++e)
 #pragma unroll
-      for (int v = 0; v < NB; ++v) {
-        __stcs(nblk + e * NB + v, neg(o.di[e][v]));
-        if (!face_zero<NB>(e, v)) sn[32 * (3 + 3 * e + v)] = o.dj[e][v];
-      }
-      if (face_flux) __stcs(face_flux + (d * NB + e) * N + c, o.F[e]);
-    }
+      for (int v = 0; v < NB; ++v) blk[e][v] = neg(o.di[e][v]);
+    store_blocks<NB>(st, blk, nbase);
   }
 }
 
 template <int NB>
-__device__ __forceinline__ void face_body(const ModelArgs& M, long long c) {
+__device__ __forceinline__ void face_body(const ModelArgs& M, long long c, bool live, WarpStage<NB>& st) {
   double r[NB], dg[NB][NB];
-  face_part<NB, false>(M, c, r, dg);
+  face_part<NB, false>(M, c, live, st, r, dg);
+  if (!live) return;
   double* s = cell_scratch(M.scr, c) + 32 * kPart;
 #pragma unroll
   for (int e = 0; e < NB; ++e) {
@@ -282,15 +336,15 @@ __device__ __forceinline__ void face_body(const ModelArgs& M, long long c) {
 
 // Row c of the residual and its diagonal block: r, dg (own terms and + faces)
 // minus the shares its - neighbours handed over, in the fixed order -z, -y,
-// -x (LinearSystem assembly, one writer per entry).
+// -x (LinearSystem assembly, one writer per entry).  Whole warps call it.
 template <int NB, bool COH>
-__device__ __forceinline__ void assemble_rows(const ModelArgs& M, long long c, double (&r)[NB],
-                                              double (&dg)[NB][NB]) {
+__device__ __forceinline__ void assemble_rows(const ModelArgs& M, long long c, bool live, WarpStage<NB>& st,
+                                              double (&r)[NB], double (&dg)[NB][NB]) {
   const Params& P = M.P;
   const double* scr = cell_scratch(M.scr, c);
   int i, j, k;
   cell_ijk(P, c, i, j, k);
-  const bool hm[3] = {i > 0, j > 0, k > 0};
+  const bool hm[3] = {live && i > 0, live && j > 0, live && k > 0};
 #pragma unroll
   for (int d = 2; d >= 0; --d) {
     if (!hm[d]) continue;
@@ -306,26 +360,42 @@ __device__ __forceinline__ void assemble_rows(const ModelArgs& M, long long c, d
   double* out = M.val + (row_start_ijk(P, c, i, j, k) + (int)hm[0] + (int)hm[1] + (int)hm[2]) * NB * NB;
   bool ok = true;
 #pragma unroll
-  for (int e = 0; e < NB; ++e) {
-    __stcs(M.res + c * NB + e, r[e]);
-    ok = ok && finite(r[e]);
-#pragma unroll
-    for (int v = 0; v < NB; ++v) __stcs(out + e * NB + v, dg[e][v]);
-  }
+  for (int e = 0; e < NB; ++e) ok = ok && (!live || finite(r[e]));
   if (!ok) atomicOr(M.status, kStatNonFinite);
+  store_blocks<NB>(st, dg, live ? out : nullptr);
+  if constexpr (NB == 3) {               // the warp's residuals are contiguous: stored in order
+    const int lane = threadIdx.x & 31;
+    const long long first = (c - lane) * NB, end = P.N * NB;
+    if (live) {
+#pragma unroll
+      for (int e = 0; e < NB; ++e) st.v[NB * lane + e] = r[e];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k3 = 0; k3 < NB; ++k3) {
+      const int q = 32 * k3 + lane;
+      if (first + q < end) __stcs(M.res + first + q, st.v[q]);
+    }
+    __syncwarp();
+  } else if (live) {
+#pragma unroll
+    for (int e = 0; e < NB; ++e) __stcs(M.res + c * NB + e, r[e]);
+  }
 }
 
 template <int NB>
-__device__ __forceinline__ void assemble_body(const ModelArgs& M, long long c) {
+__device__ __forceinline__ void assemble_body(const ModelArgs& M, long long c, bool live, WarpStage<NB>& st) {
   const double* s = cell_scratch(M.scr, c) + 32 * kPart;
   double r[NB], dg[NB][NB];
+  if (live) {
 #pragma unroll
-  for (int e = 0; e < NB; ++e) {
-    r[e] = s[32 * e];
+    for (int e = 0; e < NB; ++e) {
+      r[e] = s[32 * e];
 #pragma unroll
-    for (int v = 0; v < NB; ++v) dg[e][v] = s[32 * (3 + 3 * e + v)];
+      for (int v = 0; v < NB; ++v) dg[e][v] = s[32 * (3 + 3 * e + v)];
+    }
   }
-  assemble_rows<NB, false>(M, c, r, dg);
+  assemble_rows<NB, false>(M, c, live, st, r, dg);
 }
 
 // The model and first cell of tile t.
@@ -367,24 +437,26 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) cell_kernel(TileList L, ModelA
 template <int NB, int TPB>
 __global__ void __launch_bounds__(TPB, (NB == 3 ? 384 : 512) / TPB) face_kernel(TileList L, ModelArgs single) {
   pdl_wait();
+  __shared__ WarpStage<NB> stage[TPB / 32];
   for (int t = blockIdx.x; t < L.ntiles; t += gridDim.x) {
     int m;
     long long c0;
     const ModelArgs& M = tile_of<TPB>(L, single, t, m, c0);
     const long long c = c0 + threadIdx.x;
-    if (c < M.P.N) face_body<NB>(M, c);
+    face_body<NB>(M, c, c < M.P.N, stage[threadIdx.x >> 5]);
   }
 }
 
 template <int NB, int TPB>
 __global__ void __launch_bounds__(TPB) assemble_kernel(TileList L, ModelArgs single) {
   pdl_wait();
+  __shared__ WarpStage<NB> stage[TPB / 32];
   for (int t = blockIdx.x; t < L.ntiles; t += gridDim.x) {
     int m;
     long long c0;
     const ModelArgs& M = tile_of<TPB>(L, single, t, m, c0);
     const long long c = c0 + threadIdx.x;
-    if (c < M.P.N) assemble_body<NB>(M, c);
+    assemble_body<NB>(M, c, c < M.P.N, stage[threadIdx.x >> 5]);
   }
 }
 
@@ -1151,12 +1223,20 @@ __device__ __forceinline__ void wait_tiles(const int* flags, const long long (&l
   __syncthreads();
 }
 
+// The cell stage as a call: inlined next to the face stage, the two kernels'
+// registers together spilled a kilobyte per thread.
+template <int NB>
+__device__ __noinline__ void cell_item(const ModelArgs& M, const Table& T, long long c) {
+  cell_body<NB>(M, T, c);
+}
+
 template <int NB, int TPB, int MODE>
 __global__ void __launch_bounds__(TPB, (NB == 3 ? 384 : 512) / TPB) ordered_kernel(OrderedList O,
                                                                                     ModelArgs single) {
   pdl_wait();
   __shared__ Table T;
   __shared__ unsigned long long bar;
+  __shared__ WarpStage<NB> stage[TPB / 32];
   __shared__ long long s_tile;
   __shared__ int s_model, s_kind, s_stop;
   unsigned uses = 0;
@@ -1210,7 +1290,7 @@ __global__ void __launch_bounds__(TPB, (NB == 3 ? 384 : 512) / TPB) ordered_kern
         load_table(T, M.table, bar, uses, M.status);   // previous one: every item ends past a barrier)
         cur = mo;
       }
-      if (c < N) cell_body<NB>(M, T, c);
+      if (c < N) cell_item<NB>(M, T, c);
       __syncthreads();
       if (threadIdx.x == 0) {
         __threadfence();
@@ -1223,7 +1303,7 @@ __global__ void __launch_bounds__(TPB, (NB == 3 ? 384 : 512) / TPB) ordered_kern
       wait_tiles<TPB>(O.flag_cell + fbase, lo, hi, N, -1, M.status);
     }
     double r[NB], dg[NB][NB];
-    if (c < N) face_part<NB, MODE == 2>(M, c, r, dg);
+    face_part<NB, MODE == 2>(M, c, c < N, stage[threadIdx.x >> 5], r, dg);
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();
@@ -1233,7 +1313,7 @@ __global__ void __launch_bounds__(TPB, (NB == 3 ? 384 : 512) / TPB) ordered_kern
       const long long lo[3] = {c0 - 1, c0 - nx, c0 - nxy}, hi[3] = {c1 - 2, c1 - 1 - nx, c1 - 1 - nxy};
       wait_tiles<TPB>(O.flag_face + fbase, lo, hi, N, t, M.status);
     }
-    if (c < N) assemble_rows<NB, true>(M, c, r, dg);
+    assemble_rows<NB, true>(M, c, c < N, stage[threadIdx.x >> 5], r, dg);
     // The tile's scratch is now dead: its shares were just read, its own
     // terms in its face stage, and its cell quantities by its own face stage
     // and by the face stages of the tiles holding its cells' - neighbours,

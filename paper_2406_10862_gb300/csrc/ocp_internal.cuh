@@ -94,24 +94,24 @@ inline int tile_index(int tpb) {
     if (kTileSizes[t] == tpb) return t;
   return -1;
 }
-// Default launch shape of one grid of N cells on an SM count `sms`: the
-// largest tiles (128 for the register-heavy cell and face stages, 256 for
-// assembly) that still give every SM at least two CTAs, down to 32-cell
-// tiles; a grid too small for that (fewer than 64 cells per SM) takes the
-// face stage split by direction and the assembly by equation, since its
-// time is its warps' FP64 instruction count, not the SMs' throughput, and a
-// grid of at most `max_cluster` 32-cell tiles runs all three stages in one
-// cluster launch.
+// Default launch shape of one grid of N cells on an SM count `sms`.  One warp
+// per CTA for the face and assembly stages: their warps share nothing, and
+// the finer CTAs leave a smaller last wave (200 000 cells: 163 us, against
+// 168 with 64-cell and 173 with 128/128/256-cell tiles; 50 000: 46 against 49
+// and 50; 1 M: 750 against 755 and 763).  The cell stage's CTAs copy the PVT
+// table, so they hold 64 cells where that still gives every SM two of them.
+// Grids of fewer than four 32-cell tiles per SM take the face stage split by
+// direction and the assembly by equation, since their time is their warps'
+// FP64 instruction count, not the SMs' throughput (10 000 cells: 23 against 28
+// us; 20 000: 29 against 29; 30 000: 42 against 34), and a grid of at most
+// `max_cluster` 32-cell tiles runs all three stages in one cluster launch.
 inline LaunchCfg default_cfg(long long N, int sms, int max_cluster = 0) {
   LaunchCfg c;
   const long long S = sms > 0 ? sms : 1;
-  for (int s = 0; s < 3; ++s) {
-    int t = s < 2 ? 128 : 256;
-    while (t > 32 && N < 2LL * t * S) t /= 2;
-    c.tpb[s] = t;
-    c.ctas_per_sm[s] = 0;
-  }
-  c.ordered = N < 2LL * 32 * S ? 3 : 0;
+  c.tpb[0] = N < 2LL * 64 * S ? 32 : 64;
+  c.tpb[1] = c.tpb[2] = 32;
+  for (int s = 0; s < 3; ++s) c.ctas_per_sm[s] = 0;
+  c.ordered = N < 4LL * 32 * S ? 3 : 0;
   if (N > 0 && (N + 31) / 32 <= max_cluster) c.ordered = 4;
   return c;
 }
