@@ -421,7 +421,7 @@ ocp_status ocp_residual_norms(ocp_grid* grid, const double* residual, double dt,
  * may be NULL) also the full system, rows water, oil[, gas], volume and
  * columns P, N_w, N_o[, N_g].  flag (device int8 [N], may be NULL) receives the
  * split's state (1: undersaturated).  The first call on a grid allocates the
- * split's per-cell data (32 doubles and a byte per cell with three phases, 18
+ * split's per-cell data (24 doubles and a byte per cell with three phases, 12
  * and a byte with two), so it must not be the call captured into a CUDA
  * graph; later calls allocate nothing.  A non-finite input sets the sticky status OCP_ERR_NONFINITE. */
 ocp_status ocp_linearize_pn(ocp_grid* grid, const double* pn_new, const double* pn_old, double dt,

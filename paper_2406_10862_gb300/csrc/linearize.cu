@@ -29,8 +29,9 @@
 // device table of per-model arguments and an explicit tile list.  Both run
 // the same kernels, so a batched linearisation is bit-identical to the
 // per-grid one, whatever the tile size or the number of CTAs.
-#include "ocp_internal.cuh"
+#include "block_io.cuh"
 #include "kernels.cuh"
+#include "ocp_internal.cuh"
 
 namespace ocp {
 
@@ -193,54 +194,6 @@ __device__ __forceinline__ void cell_body(const ModelArgs& M, const Table& T, lo
     cell_terms<NB, NB == 3>(M, T, s, pn, swn, xn, 0, po, swo, xo, fo & 1, phs, ip);
   else
     cell_terms<NB, false>(M, T, s, pn, swn, xn, fn & 1, po, swo, xo, fo & 1, phs, ip);
-}
-
-// ------------------------------------------------------------ block stores
-// A warp's blocks go to the Jacobian through shared memory.  Each lane's 3x3
-// block is 72 contiguous bytes, but its neighbour lane's lies a whole row
-// (about 500 bytes) away, so one store per lane and entry touches 32 lines and
-// writes 8 bytes of each: at 200 000 cells 65 sectors a cell went through the
-// L1's store path, the loads behind them waited, and the face stage's warps
-// spent 36 % of their time on that.  Storing the 288 values in block order
-// instead, nine lanes to a block, touches four lines at a time.  A 2x2 block
-// is one 32-byte sector: a single wide store where the matrix is aligned to it.
-template <int NB>
-struct WarpStage {
-  double v[NB == 3 ? 32 * 9 : 1];
-  double* p[NB == 3 ? 32 : 1];
-};
-// Stores block b of every lane of the warp at its base (null: none).
-template <int NB>
-__device__ __forceinline__ void store_blocks(WarpStage<NB>& st, const double (&b)[NB][NB], double* base) {
-  if constexpr (NB == 3) {
-    const int lane = threadIdx.x & 31;
-    if (base) {
-#pragma unroll
-      for (int e = 0; e < 3; ++e)
-#pragma unroll
-        for (int v = 0; v < 3; ++v) st.v[9 * lane + 3 * e + v] = b[e][v];
-    }
-    st.p[lane] = base;
-    __syncwarp();
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      const int q = 32 * k + lane, r = (q * 57) >> 9;    // q / 9 for q < 288
-      double* p = st.p[r];
-      if (p) __stcs(p + (q - 9 * r), st.v[q]);
-    }
-    __syncwarp();
-  } else if (base) {
-    if (((uintptr_t)base & 31) == 0) {
-      asm volatile("st.global.cs.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(base), "d"(b[0][0]), "d"(b[0][1]), "d"(b[1][0]),
-                   "d"(b[1][1])
-                   : "memory");
-    } else {
-#pragma unroll
-      for (int e = 0; e < NB; ++e)
-#pragma unroll
-        for (int v = 0; v < NB; ++v) __stcs(base + e * NB + v, b[e][v]);
-    }
-  }
 }
 
 // The +x, +y, +z faces of cell c (BulkConn): the two off-diagonal blocks of

@@ -23,6 +23,7 @@
 //                     the volume row.
 #include <cmath>
 
+#include "block_io.cuh"
 #include "kernels.cuh"
 #include "ocp_internal.cuh"
 #include "pn_split.cuh"
@@ -30,144 +31,245 @@
 namespace ocp {
 namespace {
 
-// per-cell data of the (P, N) path, variable-major blocks of N doubles
+// Per-cell data of the (P, N) path.  First the natural state, variable-major
+// as ocp_linearize takes it; then, in tiles of 32 cells [cell / 32][field]
+// [cell % 32] (every field at a constant offset, in whole lines), T and t
+// without their first rows -- M's first row is (1, 0, ..), since p = P, so
+// T's is too and t's first entry is zero -- and, for the full system only,
+// M without its first row, the volume row a and r_v.
 template <int NB>
 struct PnLayout {
-  static constexpr int kNat = 0;                       // natural state, NB
-  static constexpr int kT = NB;                        // T, NB*NB (row-major)
-  static constexpr int kt = NB + NB * NB;              // t, NB
-  static constexpr int kM = 2 * NB + NB * NB;          // M, NB*(NB+1)
-  static constexpr int kA = kM + NB * (NB + 1);        // volume row a, NB+1, then r_v
-  static constexpr int kCount = kA + NB + 2;
+  static constexpr int kT = 0;                          // T rows 1 .., (NB - 1) NB
+  static constexpr int kt = (NB - 1) * NB;              // t entries 1 .., NB - 1
+  static constexpr int kTFields = kt + NB - 1;
+  static constexpr int kM = 0;                          // M rows 1 .., (NB - 1)(NB + 1)
+  static constexpr int kA = (NB - 1) * (NB + 1);        // a, NB + 1, then r_v
+  static constexpr int kFullFields = kA + NB + 2;
+  static __host__ __device__ long long cells(long long N) { return (N + 31) / 32 * 32; }
+  static __host__ __device__ long long tile_start(long long N) { return NB * cells(N); }
+  static __host__ __device__ long long full_start(long long N) { return tile_start(N) + kTFields * cells(N); }
+  static __host__ __device__ long long doubles(long long N) { return full_start(N) + kFullFields * cells(N); }
 };
+__device__ __forceinline__ long long tile_at(long long c, int fields) { return (c >> 5) * (32 * fields) + (c & 31); }
 
 template <int NB>
-__global__ void pn_split_kernel(Params P, const Table* __restrict__ gT, const double* __restrict__ pn,
-                                const double* __restrict__ phi_ref, double* __restrict__ d,
-                                int8_t* __restrict__ flag, double* __restrict__ elim, int* status) {
+__global__ void __launch_bounds__(128) pn_split_kernel(Params P, const Table* __restrict__ gT,
+                                                       const double* __restrict__ pn,
+                                                       const double* __restrict__ phi_ref, double* __restrict__ d,
+                                                       int8_t* __restrict__ flag, int8_t* __restrict__ flag_out,
+                                                       double* __restrict__ elim, int full, int* status) {
   using Lo = PnLayout<NB>;
   constexpr int L = NB + 1;
+  pdl_wait();
   const long long N = P.N;
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c >= N) return;
   const Table& T = *gT;
   const double p = pn[c], nw = pn[N + c], no = pn[2 * N + c], ng = (NB == 3) ? pn[3 * N + c] : 0.0;
+  const double pr = phi_ref[c];
   if (!(finite(p) && finite(nw) && finite(no) && finite(ng))) atomicOr(status, kStatNonFinite);
   Split<NB> sp;
   phase_split<NB>(P, T, p, nw, no, ng, sp);
-  const double Vf = sp.Vf;
-  const double* dVf = sp.dVf;
-  const double sw = sp.sw, x = sp.x;
-  const int f = sp.flag;
   const auto& M = sp.M;
+  d[c] = p;
+  d[N + c] = sp.sw;
+  if (NB == 3) d[2 * N + c] = sp.x;
+  if (NB == 3) flag[c] = (int8_t)sp.flag;
+  if (flag_out) flag_out[c] = NB == 3 ? (int8_t)sp.flag : (int8_t)0;
   // volume balance r_v = phi(p) - V_f and its row a
-  const double phi = phi_ref[c] * fma(P.cr, p - P.p_ref, 1.0);
-  const double rv = phi - Vf;
+  const double phi = pr * fma(P.cr, p - P.p_ref, 1.0);
+  const double rv = phi - sp.Vf;
   double a[L];
-  a[0] = phi_ref[c] * P.cr - dVf[0];
-  for (int k = 1; k < L; ++k) a[k] = -dVf[k];
+  a[0] = pr * P.cr - sp.dVf[0];
+  for (int k = 1; k < L; ++k) a[k] = -sp.dVf[k];
   // eliminate N_w: dN_w = -(c_P dP + c_o dN_o [+ c_g dN_g]) + c_r
   const double iaw = 1.0 / a[1];
   double cc[L];                         // c_P, (unused), c_o[, c_g]
   for (int k = 0; k < L; ++k) cc[k] = a[k] * iaw;
   const double cr = rv * iaw;
   // reduced columns: P, N_o[, N_g] = full columns 0, 2[, 3]
-  double* __restrict__ dp = d;
-  for (int i = 0; i < NB; ++i) {
+  double* td = d + Lo::tile_start(N) + tile_at(c, Lo::kTFields);
+#pragma unroll
+  for (int i = 1; i < NB; ++i) {
+#pragma unroll
     for (int j = 0; j < NB; ++j) {
       const int k = (j == 0) ? 0 : j + 1;
-      dp[(Lo::kT + i * NB + j) * N + c] = fma(-M[i][1], cc[k], M[i][k]);
+      td[32 * (Lo::kT + (i - 1) * NB + j)] = fma(-M[i][1], cc[k], M[i][k]);
     }
-    dp[(Lo::kt + i) * N + c] = M[i][1] * cr;
-    for (int k = 0; k < L; ++k) dp[(Lo::kM + i * L + k) * N + c] = M[i][k];
+    td[32 * (Lo::kt + i - 1)] = M[i][1] * cr;
   }
-  for (int k = 0; k < L; ++k) dp[(Lo::kA + k) * N + c] = a[k];
-  dp[(Lo::kA + L) * N + c] = rv;
-  dp[(Lo::kNat + 0) * N + c] = p;
-  dp[(Lo::kNat + 1) * N + c] = sw;
-  if (NB == 3) dp[(Lo::kNat + 2) * N + c] = x;
-  if (NB == 3) flag[c] = (int8_t)f;
+  if (full) {
+    double* fd = d + Lo::full_start(N) + tile_at(c, Lo::kFullFields);
+#pragma unroll
+    for (int i = 1; i < NB; ++i)
+#pragma unroll
+      for (int k = 0; k < L; ++k) fd[32 * (Lo::kM + (i - 1) * L + k)] = M[i][k];
+#pragma unroll
+    for (int k = 0; k < L; ++k) fd[32 * (Lo::kA + k)] = a[k];
+    fd[32 * (Lo::kA + L)] = rv;
+  }
   elim[c] = cc[0];
   elim[N + c] = cc[2];
-  if (NB == 3) elim[2 * N + c] = cc[3];
+  if (NB == 3) elim[2 * N + c] = cc[NB];
   elim[NB * N + c] = cr;
 }
 
-// The row's blocks are walked on the grid's 7-point pattern (neighbour
-// types -z, -y, -x, self, +x, +y, +z, the order of the stored columns), with
-// the row start in closed form: no dependent index loads, so every block's
-// gathers can be issued early, and the diagonal's extra terms are placed at
-// compile time.
+// One warp per 32 consecutive rows, their blocks walked on the grid's 7-point
+// pattern (neighbour types -z, -y, -x, self, +x, +y, +z, the order of the
+// stored columns), with the row start in closed form.  Blocks of one type go
+// through shared memory (block_io.cuh), the next type's on their way meanwhile:
+// read and written lane by lane, a row apart, they kept the L1 busy with 32
+// lines per access (200 000 cells: 95 us; the FP64 units' own time was 72).
+// With T's first row (1, 0, ..) and the water row's zero X column off the
+// diagonal, a 3x3 block takes 20 FMAs instead of 39.
 template <int NB>
-__global__ void __launch_bounds__(128) pn_reduce_kernel(Params P, const double* __restrict__ d,
-                                                        const double* __restrict__ elim,
-                                                        const double* __restrict__ pn_new,
-                                                        const double* __restrict__ pn_old, double scale,
-                                                        double* __restrict__ res, double* __restrict__ val,
-                                                        double* __restrict__ res4, double* __restrict__ val4) {
+__device__ __forceinline__ void reduce_block(const double (&B)[NB][NB], const double* td, bool diag, double (&out)[NB][NB],
+                                             double (&rr)[NB]) {
+  using Lo = PnLayout<NB>;
+  double Tc[NB][NB], tc[NB];
+#pragma unroll
+  for (int i = 1; i < NB; ++i) {
+#pragma unroll
+    for (int j = 0; j < NB; ++j) Tc[i][j] = td[32 * (Lo::kT + (i - 1) * NB + j)];
+    tc[i] = td[32 * (Lo::kt + i - 1)];
+  }
+#pragma unroll
+  for (int e = 0; e < NB; ++e) {
+    const int last = NB == 3 && e == 0 && !diag ? NB - 1 : NB;    // the water row's X column is zero off the diagonal
+#pragma unroll
+    for (int j = 0; j < NB; ++j) {
+      double acc = j == 0 ? B[e][0] : 0.0;
+#pragma unroll
+      for (int i = 1; i < NB; ++i)
+        if (i < last) acc = (i == 1 && j > 0) ? B[e][i] * Tc[i][j] : fma(B[e][i], Tc[i][j], acc);
+      out[e][j] = acc;
+    }
+#pragma unroll
+    for (int i = 1; i < NB; ++i)
+      if (i < last) rr[e] = fma(-B[e][i], tc[i], rr[e]);
+  }
+}
+// The block of the full system, rows water, oil[, gas], volume: B M, and the
+// volume row on the diagonal.
+template <int NB>
+__device__ __forceinline__ void full_block(const double (&B)[NB][NB], const double* fd, bool diag, double scale,
+                                           double* b4) {
   using Lo = PnLayout<NB>;
   constexpr int L = NB + 1;
+  double Mc[NB][L];
+#pragma unroll
+  for (int i = 1; i < NB; ++i)
+#pragma unroll
+    for (int k = 0; k < L; ++k) Mc[i][k] = fd[32 * (Lo::kM + (i - 1) * L + k)];
+#pragma unroll
+  for (int e = 0; e < L; ++e) {
+    double row[L];
+#pragma unroll
+    for (int k = 0; k < L; ++k) {
+      if (e == NB) {
+        row[k] = diag ? fd[32 * (Lo::kA + k)] : 0.0;
+        continue;
+      }
+      double acc = k == 0 ? B[e < NB ? e : 0][0] : 0.0;
+#pragma unroll
+      for (int i = 1; i < NB; ++i) acc = fma(B[e < NB ? e : 0][i], Mc[i][k], acc);
+      row[k] = (diag && k == e + 1) ? acc + scale : acc;
+    }
+    if constexpr (L == 4) {
+      store4(b4 + 4 * e, row);
+    } else {
+#pragma unroll
+      for (int k = 0; k < L; ++k) __stcs(b4 + L * e + k, row[k]);
+    }
+  }
+}
+
+template <int NB>
+__global__ void __launch_bounds__(32) pn_reduce_kernel(Params P, const double* __restrict__ d,
+                                                       const double* __restrict__ elim,
+                                                       const double* __restrict__ pn_new,
+                                                       const double* __restrict__ pn_old, double scale, double* res,
+                                                       double* val, double* __restrict__ res4,
+                                                       double* __restrict__ val4) {
+  using Lo = PnLayout<NB>;
+  constexpr int L = NB + 1, B2 = NB * NB;
+  pdl_wait();
+  __shared__ WarpStage<NB> st;
+  __shared__ const double* ptr[2][32];
   const long long N = P.N;
-  const long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (r >= N) return;
+  const int lane = threadIdx.x;
+  const long long r = blockIdx.x * 32ll + lane;
+  const bool live = r < N;
   int ri, rj, rk;
   cell_ijk(P, r, ri, rj, rk);
-  const bool has[7] = {rk > 0, rj > 0, ri > 0, true, ri + 1 < P.nx, rj + 1 < P.ny, rk + 1 < P.nz};
+  const bool has[7] = {live && rk > 0, live && rj > 0, live && ri > 0, live, live && ri + 1 < P.nx,
+                       live && rj + 1 < P.ny, live && rk + 1 < P.nz};
   const long long off[7] = {-P.nxy, -P.nx, -1, 0, 1, P.nx, P.nxy};
   const long long s0 = row_start_ijk(P, r, ri, rj, rk);
-  double rr[NB];
-  for (int e = 0; e < NB; ++e) rr[e] = fma(pn_new[(e + 1) * N + r] - pn_old[(e + 1) * N + r], scale, res[r * NB + e]);
-  if (res4) {
-    for (int e = 0; e < NB; ++e) res4[r * L + e] = rr[e];
-    res4[r * L + NB] = d[(Lo::kA + L) * N + r];
+  const double* tiles = d + Lo::tile_start(N);
+  const double* fulls = d + Lo::full_start(N);
+  double rr[NB], el[NB + 1];
+  if (live) {
+#pragma unroll
+    for (int e = 0; e < NB; ++e) {
+      rr[e] = fma(pn_new[(e + 1) * N + r] - pn_old[(e + 1) * N + r], scale, res[r * NB + e]);
+      el[e] = elim[e * N + r];
+    }
+    el[NB] = elim[NB * N + r];
+    if (res4) {
+#pragma unroll
+      for (int e = 0; e < NB; ++e) res4[r * L + e] = rr[e];
+      res4[r * L + NB] = fulls[tile_at(r, Lo::kFullFields) + 32 * (Lo::kA + L)];
+    }
   }
-  int slot = 0;
+  double* blk = val + s0 * B2;           // the next block of this row
+  double x[9];
+  if constexpr (NB == 3) {
+    ptr[0][lane] = has[0] ? blk : nullptr;
+    __syncwarp();
+    fetch_blocks(ptr[0], x);
+  }
 #pragma unroll
   for (int t = 0; t < 7; ++t) {
-    if (!has[t]) continue;
-    const long long s = s0 + slot;
-    ++slot;
-    const long long c = r + off[t];
-    double B[NB][NB];
-    for (int e = 0; e < NB; ++e)
-      for (int v = 0; v < NB; ++v) B[e][v] = val[(long long)s * NB * NB + e * NB + v];
-    double Tc[NB][NB], tc[NB];
-    for (int i = 0; i < NB; ++i) {
-      tc[i] = d[(Lo::kt + i) * N + c];
-      for (int j = 0; j < NB; ++j) Tc[i][j] = d[(Lo::kT + i * NB + j) * N + c];
+    double B[NB][NB], out[NB][NB];
+    double* base = has[t] ? blk : nullptr;
+    const long long slot = (blk - val) / B2;
+    if (has[t]) blk += B2;
+    if constexpr (NB == 3) {
+      put_blocks(st, x);
+      if (t < 6) ptr[(t + 1) & 1][lane] = has[t < 6 ? t + 1 : 6] ? blk : nullptr;
+      __syncwarp();
+      if (t < 6) fetch_blocks(ptr[(t + 1) & 1], x);
+#pragma unroll
+      for (int e = 0; e < 3; ++e)
+#pragma unroll
+        for (int v = 0; v < 3; ++v) B[e][v] = st.v[9 * lane + 3 * e + v];
+    } else if (has[t]) {
+      double b4[4];
+      load4(base, b4);
+      B[0][0] = b4[0]; B[0][1] = b4[1]; B[1][0] = b4[2]; B[1][1] = b4[3];
     }
-    if (val4) {
-      double Mc[NB][L];
-      for (int i = 0; i < NB; ++i)
-        for (int k = 0; k < L; ++k) Mc[i][k] = d[(Lo::kM + i * L + k) * N + c];
-      double* b4 = val4 + (long long)s * L * L;
-      for (int e = 0; e < NB; ++e)
-        for (int k = 0; k < L; ++k) {
-          double acc = 0.0;
-          for (int i = 0; i < NB; ++i) acc = fma(B[e][i], Mc[i][k], acc);
-          b4[e * L + k] = (t == 3 && k == e + 1) ? acc + scale : acc;
-        }
-      for (int k = 0; k < L; ++k) b4[NB * L + k] = (t == 3) ? d[(Lo::kA + k) * N + r] : 0.0;
-    }
-    for (int e = 0; e < NB; ++e) {
-      double corr = 0.0;
-      for (int i = 0; i < NB; ++i) corr = fma(B[e][i], tc[i], corr);
-      rr[e] -= corr;
-      for (int j = 0; j < NB; ++j) {
-        double acc = 0.0;
-        for (int i = 0; i < NB; ++i) acc = fma(B[e][i], Tc[i][j], acc);
-        if (t == 3) {
-          // accumulation (N_e - N_e,old) V/dt: water row through the
-          // eliminated N_w, the other rows on their own amounts
-          if (e == 0) acc = fma(-elim[j * N + r], scale, acc);
-          else if (j == e) acc += scale;
-        }
-        val[s * NB * NB + e * NB + j] = acc;
+    if (has[t]) {
+      const long long c = r + off[t];
+      reduce_block<NB>(B, tiles + tile_at(c, Lo::kTFields), t == 3, out, rr);
+      if (val4) full_block<NB>(B, fulls + tile_at(c, Lo::kFullFields), t == 3, scale, val4 + slot * L * L);
+      if (t == 3) {
+        // accumulation (N_e - N_e,old) V/dt: water row through the
+        // eliminated N_w, the other rows on their own amounts
+#pragma unroll
+        for (int j = 0; j < NB; ++j) out[0][j] = fma(-el[j], scale, out[0][j]);
+#pragma unroll
+        for (int e = 1; e < NB; ++e) out[e][e] += scale;
       }
     }
+    if constexpr (NB == 3) __syncwarp();   // every lane has its block before the stage is written again
+    if (__any_sync(0xffffffffu, has[t])) store_blocks<NB>(st, out, base);
   }
-  rr[0] = fma(-elim[NB * N + r], scale, rr[0]);
-  for (int e = 0; e < NB; ++e) res[r * NB + e] = rr[e];
+  if (live) {
+    rr[0] = fma(-el[NB], scale, rr[0]);
+#pragma unroll
+    for (int e = 0; e < NB; ++e) res[r * NB + e] = rr[e];
+  }
 }
 
 template <int NB>
@@ -258,8 +360,8 @@ ocp_status ocp_linearize_pn(ocp_grid* g, const double* pn_new, const double* pn_
   const long long N = g->prm.N;
   cudaError_t e = cudaSuccess;
   if (!g->d_pn) {
-    const long long per = nb == 3 ? PnLayout<3>::kCount : PnLayout<2>::kCount;
-    e = cudaMalloc((void**)&g->d_pn, sizeof(double) * per * N);
+    const long long n = nb == 3 ? PnLayout<3>::doubles(N) : PnLayout<2>::doubles(N);
+    e = cudaMalloc((void**)&g->d_pn, sizeof(double) * n);
     if (e == cudaSuccess) e = cudaMalloc((void**)&g->d_pn_flag, (size_t)N);
     if (e == cudaSuccess) e = cudaMemset(g->d_pn_flag, 0, (size_t)N);
     if (e != cudaSuccess) {
@@ -272,28 +374,28 @@ ocp_status ocp_linearize_pn(ocp_grid* g, const double* pn_new, const double* pn_
   }
   cudaStream_t s = (cudaStream_t)stream;
   const double scale = g->prm.vol_rb / dt;
+  const int full = residual_full || bsr_val_full;
   if (nb == 3)
-    pn_split_kernel<3><<<nblk(N), 256, 0, s>>>(g->prm, g->d_table, pn_new, g->d_phi, g->d_pn, g->d_pn_flag, elim,
-                                               g->d_status);
+    e = launch_pdl(pn_split_kernel<3>, nblk(N, 128), 128, 0, s, g->prm, (const Table*)g->d_table, pn_new,
+                   (const double*)g->d_phi, g->d_pn, g->d_pn_flag, flag, elim, full, g->d_status);
   else
-    pn_split_kernel<2><<<nblk(N), 256, 0, s>>>(g->prm, g->d_table, pn_new, g->d_phi, g->d_pn, g->d_pn_flag, elim,
-                                               g->d_status);
-  e = cudaGetLastError();
+    e = launch_pdl(pn_split_kernel<2>, nblk(N, 128), 128, 0, s, g->prm, (const Table*)g->d_table, pn_new,
+                   (const double*)g->d_phi, g->d_pn, g->d_pn_flag, flag, elim, full, g->d_status);
   // the natural path on the split state, accumulation left out (the natural
   // state is its own old state: nothing is read from it)
   const double* unat = g->d_pn;
   if (e == cudaSuccess)
     e = launch_linearize(g, unat, g->d_pn_flag, unat, g->d_pn_flag, dt, residual, bsr_val, nullptr, s, nullptr, 1);
   if (e == cudaSuccess) {
+    const double* pd = g->d_pn;
+    const double* el = elim;
     if (nb == 3)
-      pn_reduce_kernel<3><<<nblk(N, 128), 128, 0, s>>>(g->prm, g->d_pn, elim, pn_new,
-                                                       pn_old, scale, residual, bsr_val, residual_full, bsr_val_full);
+      e = launch_pdl(pn_reduce_kernel<3>, nblk(N, 32), 32, 0, s, g->prm, pd, el, pn_new, pn_old, scale, residual,
+                     bsr_val, residual_full, bsr_val_full);
     else
-      pn_reduce_kernel<2><<<nblk(N, 128), 128, 0, s>>>(g->prm, g->d_pn, elim, pn_new,
-                                                       pn_old, scale, residual, bsr_val, residual_full, bsr_val_full);
-    e = cudaGetLastError();
+      e = launch_pdl(pn_reduce_kernel<2>, nblk(N, 32), 32, 0, s, g->prm, pd, el, pn_new, pn_old, scale, residual,
+                     bsr_val, residual_full, bsr_val_full);
   }
-  if (e == cudaSuccess && flag) e = cudaMemcpyAsync(flag, g->d_pn_flag, (size_t)N, cudaMemcpyDeviceToDevice, s);
   if (e != cudaSuccess) return report(OCP_ERR_CUDA, "ocp_linearize_pn: %s", cudaGetErrorString(e));
   return OCP_OK;
 }
