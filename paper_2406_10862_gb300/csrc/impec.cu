@@ -25,219 +25,259 @@
 namespace ocp {
 namespace {
 
+// Per-cell data at the old level, in tiles of 32 cells [cell / 32][field]
+// [cell % 32] of the grid's scratch: every field at a constant offset from one
+// address, in whole lines.  The phase pressures are p + (p_a - p).
 enum {
-  kP = 0, kOffW, kOffG, kRhoW, kRhoO, kRhoG, kLamW, kLamO, kLamG, kRs, kWw, kWo, kWg, kDiag0, kE0, kMob, kBw, kBg,
+  kPw = 0, kPo, kPg, kLamW, kLamO, kLamG, kRs, kRhoW, kRhoO, kRhoG, kWw, kWo, kWg, kDiag0, kE0, kMob, kBw, kBg,
   kImpecSlots
 };
+__device__ __forceinline__ long long impec_at(long long c) { return (c >> 5) * (32 * kImpecSlots) + (c & 31); }
 
 template <int NB>
-__global__ void impec_cell_kernel(Params P, const Table* __restrict__ gT, const double* __restrict__ pn,
-                                  const double* __restrict__ phi_ref, double scale, double* __restrict__ d,
-                                  int* status) {
+__global__ void __launch_bounds__(128) impec_cell_kernel(Params P, const Table* __restrict__ gT,
+                                                         const double* __restrict__ pn,
+                                                         const double* __restrict__ phi_ref,
+                                                         const int32_t* __restrict__ perf_of_cell, double scale,
+                                                         double* __restrict__ scratch, int* status) {
+  pdl_wait();
+  __shared__ Table T;
+  __shared__ unsigned long long bar;
+  unsigned uses = 0;
+  load_table(T, gT, bar, uses, status);
   const long long N = P.N;
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c >= N) return;
   const double p = pn[c], nw = pn[N + c], no = pn[2 * N + c], ng = (NB == 3) ? pn[3 * N + c] : 0.0;
+  const double pr = phi_ref[c];
+  const int ip = perf_of_cell[c];
   if (!(finite(p) && finite(nw) && finite(no) && finite(ng))) atomicOr(status, kStatNonFinite);
   Split<NB> sp;
-  phase_split<NB>(P, *gT, p, nw, no, ng, sp);
+  phase_split<NB>(P, T, p, nw, no, ng, sp);
   CellQ q{};
   CellAux a{};
-  cell_quantities<NB, true>(P, *gT, p, sp.sw, sp.x, sp.flag, phi_ref[c], q, a, true);
-  const double phi = phi_ref[c] * fma(P.cr, p - P.p_ref, 1.0);
-  d[kP * N + c] = p;
-  d[kOffW * N + c] = q.pw - p;
-  d[kOffG * N + c] = (NB == 3) ? q.pg - p : 0.0;
-  d[kRhoW * N + c] = q.rw;
-  d[kRhoO * N + c] = q.ro;
-  d[kRhoG * N + c] = (NB == 3) ? q.rg : 0.0;
-  d[kLamW * N + c] = q.lw;
-  d[kLamO * N + c] = q.lo;
-  d[kLamG * N + c] = (NB == 3) ? q.lg : 0.0;
-  d[kRs * N + c] = (NB == 3) ? q.rs : 0.0;
-  d[kWw * N + c] = sp.dVf[1];
-  d[kWo * N + c] = sp.dVf[2];
-  d[kWg * N + c] = (NB == 3) ? sp.dVf[3] : 0.0;
-  d[kDiag0 * N + c] = scale * (phi_ref[c] * P.cr - sp.dVf[0]);
-  d[kE0 * N + c] = scale * (phi - sp.Vf);
-  d[kMob * N + c] = a.mob;
-  d[kBw * N + c] = a.bw;
-  d[kBg * N + c] = (NB == 3) ? a.bg : 0.0;
-}
-
-// The cell's neighbours in column order (-z, -y, -x, +x, +y, +z) and the
-// data of one face: per phase the frozen coefficient T lambda_up and the old
-// potential difference (from the cell to the neighbour), and the oil's
-// upwind R_s.
-struct FaceCoef {
-  double c[3], dphi[3], rs_up;
-};
-
-template <int NB>
-__device__ __forceinline__ void face_coef(const Params& P, const double* __restrict__ d, long long c, long long n,
-                                          double T, double hz, FaceCoef& f) {
-  const long long N = P.N;
-  const double pc = d[kP * N + c], pn_ = d[kP * N + n];
-  const int offs[3] = {kOffW, -1, kOffG};
-  const int rhos[3] = {kRhoW, kRhoO, kRhoG};
-  const int lams[3] = {kLamW, kLamO, kLamG};
-  for (int ph = 0; ph < NB; ++ph) {                // water, oil[, gas]
-    const int al = ph;
-    const double oc = offs[ph] >= 0 ? d[offs[ph] * N + c] : 0.0;
-    const double on = offs[ph] >= 0 ? d[offs[ph] * N + n] : 0.0;
-    double dphi = (pc + oc) - (pn_ + on);
-    if (hz != 0.0) dphi = fma(-(d[rhos[ph] * N + c] + d[rhos[ph] * N + n]), hz, dphi);
-    const bool up = nonneg(dphi);
-    f.c[al] = T * (up ? d[lams[ph] * N + c] : d[lams[ph] * N + n]);
-    f.dphi[al] = dphi;
-    if (al == 1) f.rs_up = (NB == 3) ? (up ? d[kRs * N + c] : d[kRs * N + n]) : 0.0;
-  }
-}
-
-// Neighbour t of c (t = 0..5: -z, -y, -x, +x, +y, +z): index, face axis and
-// side, transmissibility and the gravity head factor.
-__device__ __forceinline__ bool neighbour(const Params& P, const double* __restrict__ trans, long long c, int i, int j,
-                                          int k, int t, long long& n, double& T, double& hz) {
-  const int axis[6] = {2, 1, 0, 0, 1, 2};
-  const bool plus = t >= 3;
-  const int ax = axis[t];
-  bool has;
-  long long off;
-  if (ax == 0) { has = plus ? (i + 1 < P.nx) : (i > 0); off = 1; }
-  else if (ax == 1) { has = plus ? (j + 1 < P.ny) : (j > 0); off = P.nx; }
-  else { has = plus ? (k + 1 < P.nz) : (k > 0); off = P.nxy; }
-  if (!has) return false;
-  n = plus ? c + off : c - off;
-  T = trans[ax * P.N + (plus ? c : n)];
-  hz = (ax == 2) ? (plus ? -P.grav_dz : P.grav_dz) : 0.0;
-  return true;
-}
-
-// Component fluxes out of c through one face at a pressure change
-// (dPc, dPn); K = the old-level part, C = the coefficient of (dPc - dPn).
-template <int NB>
-__device__ __forceinline__ void comp_flux(const FaceCoef& f, double* C, double* K) {
-  C[0] = f.c[0];
-  K[0] = f.c[0] * f.dphi[0];
-  C[1] = f.c[1];
-  K[1] = f.c[1] * f.dphi[1];
+  cell_quantities<NB, true>(P, T, p, sp.sw, sp.x, sp.flag, pr, q, a, ip >= 0);
+  const double phi = pr * fma(P.cr, p - P.p_ref, 1.0);
+  double* d = scratch + impec_at(c);
+  d[32 * kPw] = p + (q.pw - p);
+  d[32 * kPo] = p;
+  d[32 * kLamW] = q.lw;
+  d[32 * kLamO] = q.lo;
+  d[32 * kRhoW] = q.rw;
+  d[32 * kRhoO] = q.ro;
+  d[32 * kWw] = sp.dVf[1];
+  d[32 * kWo] = sp.dVf[2];
   if (NB == 3) {
-    C[2] = fma(f.rs_up, f.c[1], f.c[2]);
-    K[2] = fma(f.rs_up, K[1], f.c[2] * f.dphi[2]);
+    d[32 * kPg] = p + (q.pg - p);
+    d[32 * kLamG] = q.lg;
+    d[32 * kRs] = q.rs;
+    d[32 * kRhoG] = q.rg;
+    d[32 * kWg] = sp.dVf[NB];
   }
+  d[32 * kDiag0] = scale * (pr * P.cr - sp.dVf[0]);
+  d[32 * kE0] = scale * (phi - sp.Vf);
+  if (ip >= 0) {                         // read for perforated cells only
+    d[32 * kMob] = a.mob;
+    d[32 * kBw] = a.bw;
+    if (NB == 3) d[32 * kBg] = a.bg;
+  }
+}
+
+// What the faces of a cell need of it: phase pressures, mobilities, the
+// dissolved-gas ratio and, for vertical faces, the densities.
+template <int NB>
+struct ImpecSide {
+  double p[NB], l[NB], rs, rho[NB];
+};
+template <int NB>
+__device__ __forceinline__ void impec_load(const double* d, bool z, ImpecSide<NB>& f) {
+#pragma unroll
+  for (int ph = 0; ph < NB; ++ph) {
+    f.p[ph] = d[32 * (kPw + ph)];
+    f.l[ph] = d[32 * (kLamW + ph)];
+    f.rho[ph] = z ? d[32 * (kRhoW + ph)] : 0.0;
+  }
+  f.rs = NB == 3 ? d[32 * kRs] : 0.0;
+}
+
+// One face from the row cell (c) to its neighbour (n): per phase the frozen
+// coefficient T lambda_up and the old potential difference, and the oil's
+// upwind R_s.
+template <int NB>
+struct FaceCoef {
+  double c[NB], dphi[NB], rs_up;
+};
+template <int NB>
+__device__ __forceinline__ void face_coef(const ImpecSide<NB>& c, const ImpecSide<NB>& n, bool z, double T, double hz,
+                                          FaceCoef<NB>& f) {
+  f.rs_up = 0.0;
+#pragma unroll
+  for (int ph = 0; ph < NB; ++ph) {                // water, oil[, gas]
+    double dphi = c.p[ph] - n.p[ph];
+    if (z) dphi = fma(-(c.rho[ph] + n.rho[ph]), hz, dphi);
+    const bool up = nonneg(dphi);
+    f.c[ph] = T * sel(up, c.l[ph], n.l[ph]);
+    f.dphi[ph] = dphi;
+    if (ph == 1 && NB == 3) f.rs_up = sel(up, c.rs, n.rs);
+  }
+}
+
+// Neighbour t of c (t = 0..5: -z, -y, -x, +x, +y, +z) and where its face's
+// transmissibility stands.
+__device__ __forceinline__ bool neighbour(const Params& P, long long c, int i, int j, int k, int t, long long& n,
+                                          long long& face) {
+  const bool has[6] = {k > 0, j > 0, i > 0, i + 1 < P.nx, j + 1 < P.ny, k + 1 < P.nz};
+  const long long off[6] = {-P.nxy, -P.nx, -1, 1, P.nx, P.nxy};
+  const int axis = t < 3 ? 2 - t : t - 3;
+  n = c + off[t];
+  face = axis * P.N + (t < 3 ? n : c);
+  return has[t];
 }
 
 // Well terms of the cell: Q_i(dP) = Q0_i + Qp_i dP (old mobilities, open
 // state of the old level).
 template <int NB>
-__device__ __forceinline__ void well_terms(const Params& P, const double* __restrict__ d, long long c, const Perf& w,
-                                           double* Q0, double* Qp) {
-  const long long N = P.N;
+__device__ __forceinline__ void well_terms(const double* d, const Perf& w, double* Q0, double* Qp) {
   for (int e = 0; e < NB; ++e) Q0[e] = Qp[e] = 0.0;
-  const double p = d[kP * N + c];
+  const double p = d[32 * kPo];
   if (w.kind == 0) {
     if (!positive(p - w.p_bh)) return;
     const double g = w.p_bh - p;
-    const double lw = w.wi * d[kLamW * N + c], lo = w.wi * d[kLamO * N + c];
+    const double lw = w.wi * d[32 * kLamW], lo = w.wi * d[32 * kLamO];
     Q0[0] = lw * g;
     Qp[0] = neg(lw);
     Q0[1] = lo * g;
     Qp[1] = neg(lo);
     if (NB == 3) {
-      const double lg = w.wi * d[kLamG * N + c], rs = d[kRs * N + c];
-      Q0[2] = fma(rs, Q0[1], lg * g);
-      Qp[2] = neg(fma(rs, lo, lg));
+      const double lg = w.wi * d[32 * kLamG], rs = d[32 * kRs];
+      Q0[NB - 1] = fma(rs, Q0[1], lg * g);
+      Qp[NB - 1] = neg(fma(rs, lo, lg));
     }
   } else {
     if (!positive(w.p_bh - p)) return;
     const int e = (w.phase == 0) ? 0 : NB - 1;
-    const double coef = w.wi * d[kMob * N + c] * ((w.phase == 0) ? d[kBw * N + c] : d[kBg * N + c]);
+    const double coef = w.wi * d[32 * kMob] * ((w.phase == 0) ? d[32 * kBw] : d[32 * kBg]);
     Q0[e] = coef * (w.p_bh - p);
     Qp[e] = neg(coef);
   }
 }
 
+// One warp per 32 consecutive rows; their values are contiguous in val and
+// leave through shared memory in order (lane by lane they were 56 bytes
+// apart, and gathered in indexed local arrays first: 200 000 cells 70 us).
 template <int NB>
-__global__ void impec_matrix_kernel(Params P, const double* __restrict__ trans, const int32_t* __restrict__ row_ptr,
-                                    const int32_t* __restrict__ perf_of_cell, const Perf* __restrict__ perf,
-                                    const double* __restrict__ d, double* __restrict__ val, double* __restrict__ rhs) {
+__global__ void __launch_bounds__(32) impec_matrix_kernel(Params P, const double* __restrict__ trans,
+                                                          const int32_t* __restrict__ perf_of_cell,
+                                                          const Perf* __restrict__ perf,
+                                                          const double* __restrict__ scratch,
+                                                          double* __restrict__ val, double* __restrict__ rhs) {
+  pdl_wait();
+  __shared__ double out[32 * 7];
   const long long N = P.N;
-  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (c >= N) return;
-  int i, j, k;
+  const int lane = threadIdx.x;
+  const long long c0 = blockIdx.x * 32ll, c = c0 + lane;
+  const bool live = c < N;
+  int i, j, k, i0, j0, k0;
   cell_ijk(P, c, i, j, k);
-  const double w[3] = {d[kWw * N + c], d[kWo * N + c], NB == 3 ? d[kWg * N + c] : 0.0};
-  double diag = d[kDiag0 * N + c];
-  double E = d[kE0 * N + c];
-  int s = row_ptr[c];
-  double lower[3];
-  int nl = 0;
-  double upper[3];
-  int nu = 0;
-  for (int t = 0; t < 6; ++t) {
-    long long n;
-    double T, hz;
-    if (!neighbour(P, trans, c, i, j, k, t, n, T, hz)) continue;
-    FaceCoef f;
-    face_coef<NB>(P, d, c, n, T, hz, f);
-    double C[3], K[3];
-    comp_flux<NB>(f, C, K);
-    double sc = 0.0, sk = 0.0;
-    for (int e = 0; e < NB; ++e) {
-      sc = fma(w[e], C[e], sc);
-      sk = fma(w[e], K[e], sk);
+  cell_ijk(P, c0, i0, j0, k0);
+  const long long s0 = row_start_ijk(P, c0, i0, j0, k0);
+  int at = 0, count = 0;
+  if (live) {
+    at = (int)(row_start_ijk(P, c, i, j, k) - s0);
+    const double* d = scratch + impec_at(c);
+    ImpecSide<NB> own;
+    impec_load<NB>(d, true, own);
+    const double w[3] = {d[32 * kWw], d[32 * kWo], NB == 3 ? d[32 * kWg] : 0.0};
+    double diag = d[32 * kDiag0], E = d[32 * kE0];
+    const int ip = perf_of_cell[c];
+    const int below = (k > 0) + (j > 0) + (i > 0);       // place of the diagonal in the row
+    count = below + 1 + (i + 1 < P.nx) + (j + 1 < P.ny) + (k + 1 < P.nz);
+    int slot = at;
+#pragma unroll
+    for (int t = 0; t < 6; ++t) {
+      if (t == 3) ++slot;
+      long long n, face;
+      if (!neighbour(P, c, i, j, k, t, n, face)) continue;
+      const bool z = t == 0 || t == 5;
+      ImpecSide<NB> nb;
+      impec_load<NB>(scratch + impec_at(n), z, nb);
+      FaceCoef<NB> f;
+      face_coef<NB>(own, nb, z, trans[face], t == 0 ? P.grav_dz : -P.grav_dz, f);
+      // weights of the phase fluxes in the row: w_w, w_o + R_s w_g, w_g
+      double a[NB];
+      a[0] = f.c[0] * w[0];
+      a[1] = f.c[1] * (NB == 3 ? fma(w[2], f.rs_up, w[1]) : w[1]);
+      if (NB == 3) a[NB - 1] = f.c[NB - 1] * w[2];
+      double sc = a[0] + a[1], sk = fma(a[1], f.dphi[1], a[0] * f.dphi[0]);
+      if (NB == 3) {
+        sc += a[NB - 1];
+        sk = fma(a[NB - 1], f.dphi[NB - 1], sk);
+      }
+      E += sk;
+      diag += sc;
+      out[slot++] = neg(sc);
     }
-    E += sk;
-    diag += sc;
-    if (t < 3) lower[nl++] = neg(sc);
-    else upper[nu++] = neg(sc);
-  }
-  const int ip = perf_of_cell[c];
-  if (ip >= 0) {
-    double Q0[3], Qp[3];
-    well_terms<NB>(P, d, c, perf[ip], Q0, Qp);
-    for (int e = 0; e < NB; ++e) {
-      E = fma(-w[e], Q0[e], E);
-      diag = fma(-w[e], Qp[e], diag);
+    if (ip >= 0) {
+      double Q0[3], Qp[3];
+      well_terms<NB>(d, perf[ip], Q0, Qp);
+      for (int e = 0; e < NB; ++e) {
+        E = fma(-w[e], Q0[e], E);
+        diag = fma(-w[e], Qp[e], diag);
+      }
     }
+    out[at + below] = diag;
+    rhs[c] = neg(E);
   }
-  for (int q = 0; q < nl; ++q) val[s++] = lower[q];
-  val[s++] = diag;
-  for (int q = 0; q < nu; ++q) val[s++] = upper[q];
-  rhs[c] = neg(E);
+  const int last = (int)(N - 1 - c0 < 31 ? N - 1 - c0 : 31);
+  const int total = __shfl_sync(0xffffffffu, at + count, last);
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < 7; ++q)
+    if (32 * q + lane < total) val[s0 + 32 * q + lane] = out[32 * q + lane];
 }
 
 template <int NB>
-__global__ void impec_update_kernel(Params P, const double* __restrict__ trans, const int32_t* __restrict__ perf_of_cell,
-                                    const Perf* __restrict__ perf, const double* __restrict__ d,
-                                    const double* __restrict__ pn_old, const double* __restrict__ dp, double inv_scale,
-                                    double* __restrict__ pn_new) {
+__global__ void __launch_bounds__(64) impec_update_kernel(Params P, const double* __restrict__ trans,
+                                                          const int32_t* __restrict__ perf_of_cell,
+                                                          const Perf* __restrict__ perf,
+                                                          const double* __restrict__ scratch,
+                                                          const double* __restrict__ pn_old,
+                                                          const double* __restrict__ dp, double inv_scale,
+                                                          double* __restrict__ pn_new) {
+  pdl_wait();
   const long long N = P.N;
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c >= N) return;
   int i, j, k;
   cell_ijk(P, c, i, j, k);
   const double dpc = dp[c];
+  const double* d = scratch + impec_at(c);
+  ImpecSide<NB> own;
+  impec_load<NB>(d, true, own);
+  const int ip = perf_of_cell[c];
   double out[3] = {0.0, 0.0, 0.0};
+#pragma unroll
   for (int t = 0; t < 6; ++t) {
-    long long n;
-    double T, hz;
-    if (!neighbour(P, trans, c, i, j, k, t, n, T, hz)) continue;
-    FaceCoef f;
-    face_coef<NB>(P, d, c, n, T, hz, f);
+    long long n, face;
+    if (!neighbour(P, c, i, j, k, t, n, face)) continue;
+    const bool z = t == 0 || t == 5;
+    ImpecSide<NB> nb;
+    impec_load<NB>(scratch + impec_at(n), z, nb);
+    FaceCoef<NB> f;
+    face_coef<NB>(own, nb, z, trans[face], t == 0 ? P.grav_dz : -P.grav_dz, f);
     const double dd = dpc - dp[n];
     // phase fluxes at the new pressure, then components (dissolved gas with the oil)
-    double F[3];
+    double F[NB];
+#pragma unroll
     for (int al = 0; al < NB; ++al) F[al] = f.c[al] * (f.dphi[al] + dd);
     out[0] += F[0];
     out[1] += F[1];
-    if (NB == 3) out[2] += fma(f.rs_up, F[1], F[2]);
+    if (NB == 3) out[2] += fma(f.rs_up, F[1], F[NB - 1]);
   }
   double Q[3] = {0.0, 0.0, 0.0};
-  const int ip = perf_of_cell[c];
   if (ip >= 0) {
     double Q0[3], Qp[3];
-    well_terms<NB>(P, d, c, perf[ip], Q0, Qp);
+    well_terms<NB>(d, perf[ip], Q0, Qp);
     for (int e = 0; e < NB; ++e) Q[e] = fma(Qp[e], dpc, Q0[e]);
   }
   pn_new[c] = pn_old[c] + dpc;
@@ -268,22 +308,20 @@ ocp_status ocp_impec_pressure(ocp_grid* g, const double* pn, double dt, double* 
   using namespace ocp;
   if (!g || !pn || !val || !rhs) return report(OCP_ERR_INVALID_ARG, "grid, pn, val and rhs are required");
   if (!(std::isfinite(dt) && dt > 0.0)) return report(OCP_ERR_INVALID_ARG, "dt must be finite and > 0");
-  static_assert(kImpecSlots <= 100, "IMPEC data must fit the linearisation scratch");
+  static_assert(kImpecSlots <= 85, "IMPEC data must fit the linearisation scratch");
   Guard guard(g->device);
   if (guard.err != cudaSuccess) return report(OCP_ERR_CUDA, "cudaSetDevice: %s", cudaGetErrorString(guard.err));
   cudaStream_t s = (cudaStream_t)stream;
   const long long N = g->prm.N;
   const double scale = g->prm.vol_rb / dt;
-  if (g->prm.nb == 3) {
-    impec_cell_kernel<3><<<nblk(N), 256, 0, s>>>(g->prm, g->d_table, pn, g->d_phi, scale, g->d_scratch, g->d_status);
-    impec_matrix_kernel<3><<<nblk(N), 256, 0, s>>>(g->prm, g->d_trans, g->d_row_ptr, g->d_perf_of_cell, g->d_perf,
-                                                   g->d_scratch, val, rhs);
-  } else {
-    impec_cell_kernel<2><<<nblk(N), 256, 0, s>>>(g->prm, g->d_table, pn, g->d_phi, scale, g->d_scratch, g->d_status);
-    impec_matrix_kernel<2><<<nblk(N), 256, 0, s>>>(g->prm, g->d_trans, g->d_row_ptr, g->d_perf_of_cell, g->d_perf,
-                                                   g->d_scratch, val, rhs);
-  }
-  cudaError_t e = cudaGetLastError();
+  const auto cell = g->prm.nb == 3 ? impec_cell_kernel<3> : impec_cell_kernel<2>;
+  const auto matrix = g->prm.nb == 3 ? impec_matrix_kernel<3> : impec_matrix_kernel<2>;
+  cudaError_t e = launch_pdl(cell, nblk(N, 128), 128, 0, s, g->prm, (const Table*)g->d_table, pn,
+                             (const double*)g->d_phi, (const int32_t*)g->d_perf_of_cell, scale, g->d_scratch,
+                             g->d_status);
+  if (e == cudaSuccess)
+    e = launch_pdl(matrix, nblk(N, 32), 32, 0, s, g->prm, (const double*)g->d_trans,
+                   (const int32_t*)g->d_perf_of_cell, (const Perf*)g->d_perf, (const double*)g->d_scratch, val, rhs);
   if (e != cudaSuccess) return report(OCP_ERR_CUDA, "ocp_impec_pressure: %s", cudaGetErrorString(e));
   return OCP_OK;
 }
@@ -299,13 +337,10 @@ ocp_status ocp_impec_update(ocp_grid* g, const double* pn_old, const double* dp,
   cudaStream_t s = (cudaStream_t)stream;
   const long long N = g->prm.N;
   const double inv_scale = dt / g->prm.vol_rb;
-  if (g->prm.nb == 3)
-    impec_update_kernel<3><<<nblk(N), 256, 0, s>>>(g->prm, g->d_trans, g->d_perf_of_cell, g->d_perf, g->d_scratch,
-                                                   pn_old, dp, inv_scale, pn_new);
-  else
-    impec_update_kernel<2><<<nblk(N), 256, 0, s>>>(g->prm, g->d_trans, g->d_perf_of_cell, g->d_perf, g->d_scratch,
-                                                   pn_old, dp, inv_scale, pn_new);
-  cudaError_t e = cudaGetLastError();
+  const auto update = g->prm.nb == 3 ? impec_update_kernel<3> : impec_update_kernel<2>;
+  cudaError_t e = launch_pdl(update, nblk(N, 64), 64, 0, s, g->prm, (const double*)g->d_trans,
+                             (const int32_t*)g->d_perf_of_cell, (const Perf*)g->d_perf, (const double*)g->d_scratch,
+                             pn_old, dp, inv_scale, pn_new);
   if (e != cudaSuccess) return report(OCP_ERR_CUDA, "ocp_impec_update: %s", cudaGetErrorString(e));
   return OCP_OK;
 }
