@@ -30,6 +30,15 @@ __device__ __forceinline__ void load4(const double* base, double (&x)[4]) {
     for (int k = 0; k < 4; ++k) x[k] = base[k];
   }
 }
+// The same for data no one writes during the kernel.
+__device__ __forceinline__ void load4_const(const double* base, double (&x)[4]) {
+  if (((uintptr_t)base & 31) == 0) {
+    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(x[0]), "=d"(x[1]), "=d"(x[2]), "=d"(x[3]) : "l"(base));
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = __ldg(base + k);
+  }
+}
 __device__ __forceinline__ void store4(double* base, const double (&x)[4]) {
   if (((uintptr_t)base & 31) == 0) {
     asm volatile("st.global.cs.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(base), "d"(x[0]), "d"(x[1]), "d"(x[2]), "d"(x[3])

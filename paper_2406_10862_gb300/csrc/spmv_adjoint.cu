@@ -16,8 +16,9 @@
 //                   and the block-CSR pattern.
 // well_rate_kernel  surface rates of each well (one thread per well, its
 //                   perforations summed in order).
-#include "ocp_internal.cuh"
+#include "block_io.cuh"
 #include "kernels.cuh"
+#include "ocp_internal.cuh"
 
 namespace ocp {
 
@@ -147,26 +148,23 @@ __global__ void __launch_bounds__(kSpmvThreads, kSpmvMinBlocks) spmv_grid_kernel
   }
 }
 
-// Transposed product on the grid's pattern, one thread per output row c:
-// y_c = sum over the stored blocks (n, c) of A(n, c)^T x_n, with the blocks
-// visited in the order of row c's columns (neighbour types -z .. +z).  Block
-// (n, c) lies in row n at the slot of the opposite type 6 - t: n's row start
-// in closed form plus the number of n's neighbour types before 6 - t, so no
-// index is loaded.  The FMAs run in the order of a gather of row c's
-// columns: block by block, each block's rows in turn.
+// acc = A(., c)^T x over the stored blocks (n, c) of column c, visited in the
+// order of row c's columns (neighbour types -z .. +z).  Block (n, c) lies in
+// row n at the slot of the opposite type 6 - t: n's row start in closed form
+// plus the number of n's neighbour types before 6 - t, so no index is loaded.
+// The FMAs run block by block, each block's rows in turn.  A 2x2 block is one
+// wide load where it is aligned (1 122 000 rows 72.7 -> 63.8 us); the nine
+// loads of a 3x3 block hit L1 after the first, and bringing them through
+// shared memory in block order, as the linearisation stores them, measured
+// slower (200 000 rows 29.0 against 26.1 us).
 template <int NB>
-__global__ void __launch_bounds__(kSpmvThreads) spmv_grid_t_kernel(Params P, const double* __restrict__ val,
-                                                                   double alpha, const double* __restrict__ x,
-                                                                   double beta, double* __restrict__ y, int mode) {
+__device__ __forceinline__ void column_product(const Params& P, long long c, const double* __restrict__ val,
+                                               const double* __restrict__ x, double (&acc)[NB]) {
   constexpr int B2 = NB * NB;
-  pdl_wait();
-  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (c >= P.N) return;
   int ci, cj, ck;
   cell_ijk(P, c, ci, cj, ck);
   const bool has[7] = {ck > 0, cj > 0, ci > 0, true, ci + 1 < P.nx, cj + 1 < P.ny, ck + 1 < P.nz};
   const long long off[7] = {-P.nxy, -P.nx, -1, 0, 1, P.nx, P.nxy};
-  double acc[NB];
 #pragma unroll
   for (int v = 0; v < NB; ++v) acc[v] = 0.0;
 #pragma unroll
@@ -180,13 +178,32 @@ __global__ void __launch_bounds__(kSpmvThreads) spmv_grid_t_kernel(Params P, con
 #pragma unroll
     for (int u = 0; u < 6 - t; ++u) sn += hn[u];
     const double* blk = val + (row_start_ijk(P, n, ni, nj, nk) + sn) * B2;
+    double b[B2];
+    if constexpr (NB == 2) {
+      load4_const(blk, b);
+    } else {
+#pragma unroll
+      for (int q = 0; q < B2; ++q) b[q] = __ldg(blk + q);
+    }
 #pragma unroll
     for (int e = 0; e < NB; ++e) {
       const double l = x[n * NB + e];
 #pragma unroll
-      for (int v = 0; v < NB; ++v) acc[v] = fma(__ldg(blk + e * NB + v), l, acc[v]);
+      for (int v = 0; v < NB; ++v) acc[v] = fma(b[e * NB + v], l, acc[v]);
     }
   }
+}
+
+// Transposed product on the grid's pattern: y = alpha A^T x + beta y.
+template <int NB>
+__global__ void __launch_bounds__(kSpmvThreads) spmv_grid_t_kernel(Params P, const double* __restrict__ val,
+                                                                   double alpha, const double* __restrict__ x,
+                                                                   double beta, double* __restrict__ y, int mode) {
+  pdl_wait();
+  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (c >= P.N) return;
+  double acc[NB];
+  column_product<NB>(P, c, val, x, acc);
 #pragma unroll
   for (int v = 0; v < NB; ++v) {
     double o = acc[v];
@@ -235,11 +252,11 @@ template <int NB>
 constexpr int bulk_smem_bytes() { return kBulkRows * 7 * 8 * NB * NB + 16; }
 
 template <int NB>
-__global__ void __launch_bounds__(kBulkRows) spmv_bulk_kernel(Params P, const int32_t* __restrict__ row_ptr,
-                                                              long long nnzb, const double* __restrict__ val,
-                                                              double alpha, const double* __restrict__ x,
-                                                              double beta, double* __restrict__ y, int mode,
-                                                              int* __restrict__ status) {
+__global__ void __launch_bounds__(kBulkRows) spmv_bulk_kernel(Params P, long long nnzb,
+                                                                    const double* __restrict__ val, double alpha,
+                                                                    const double* __restrict__ x, double beta,
+                                                                    double* __restrict__ y, int mode,
+                                                                    int* __restrict__ status) {
   constexpr int B2 = NB * NB;
   constexpr long long BB = 8 * B2;
   pdl_wait();
@@ -247,7 +264,7 @@ __global__ void __launch_bounds__(kBulkRows) spmv_bulk_kernel(Params P, const in
   __shared__ __align__(8) unsigned long long bar;
   const long long r0 = (long long)blockIdx.x * kBulkRows;
   const long long r1 = r0 + kBulkRows < P.N ? r0 + kBulkRows : P.N;
-  const long long b0 = row_ptr[r0], b1 = row_ptr[r1];
+  const long long b0 = row_start(P, r0), b1 = row_start(P, r1);
   const long long s = (b0 * BB) & ~15ll;
   const long long end16 = (nnzb * BB) & ~15ll;
   long long e = (b1 * BB + 15) & ~15ll;
@@ -289,23 +306,22 @@ __global__ void __launch_bounds__(kBulkRows) spmv_bulk_kernel(Params P, const in
     return;
   }
   if (!live) return;
-  const double* sm = reinterpret_cast<const double*>(sbuf);
+  const double* sm = reinterpret_cast<const double*>(sbuf) - (s >> 3);    // sm[q] is val[q]
   const long long rs = row_start_ijk(P, c, ci, cj, ck);
   double acc[NB];
 #pragma unroll
   for (int q = 0; q < NB; ++q) acc[q] = 0.0;
-  int slot = 0;
+  // the array's last double may lie past the copy (odd size)
+  const double last = c == P.N - 1 && nnzb * BB > e ? val[nnzb * B2 - 1] : 0.0;
+  const double* row = sm + rs * B2;
 #pragma unroll
   for (int t = 0; t < 7; ++t) {
     if (!has[t]) continue;
-    const long long q0 = (rs + slot) * B2;   // index of the block's first double in val
-    ++slot;
     double b[B2];
 #pragma unroll
-    for (int q = 0; q < B2; ++q) {
-      const long long gi = q0 + q;
-      b[q] = gi * 8 < e ? sm[(gi * 8 - s) >> 3] : val[gi];
-    }
+    for (int q = 0; q < B2; ++q) b[q] = row[q];
+    row += B2;
+    if (c == P.N - 1 && (row - sm) * 8 > e) b[B2 - 1] = last;
 #pragma unroll
     for (int q = 0; q < NB; ++q)
 #pragma unroll
@@ -321,10 +337,11 @@ __global__ void __launch_bounds__(kBulkRows) spmv_bulk_kernel(Params P, const in
 }
 
 // ------------------------------------------------------------------ adjoint
-// 128-thread CTAs: at 64 registers four 256-thread CTAs fit an SM and the
-// 200 000-cell adjoint's 782 CTAs split 3 : 2 over the SMs; 1563 CTAs of 128
-// spread evenly enough (79 against 84 us).
-constexpr int kVjpThreads = 128;
+// One-warp CTAs with the PVT table read through L1: with a copy of the table in
+// shared memory they cost a copy per warp, and larger CTAs a coarser last wave
+// (100 000 cells: 39 us, against 40 and 43 with 64 and 128 threads and 44 with
+// 128 threads and the copy).
+constexpr int kVjpThreads = 32;
 
 template <int NB>
 __global__ void __launch_bounds__(kVjpThreads) vjp_kernel(Params P, const Table* __restrict__ gT,
@@ -340,13 +357,9 @@ __global__ void __launch_bounds__(kVjpThreads) vjp_kernel(Params P, const Table*
                                                   const Perf* __restrict__ perf, double scale,
                                                   const double* __restrict__ lam,
                                                   double* __restrict__ g_unew, double* __restrict__ g_uold,
-                                                  double* __restrict__ g_lnk, double* __restrict__ g_phi,
-                                                  int* __restrict__ status) {
+                                                  double* __restrict__ g_lnk, double* __restrict__ g_phi) {
   pdl_wait();
-  __shared__ Table T;
-  __shared__ unsigned long long bar;
-  unsigned uses = 0;
-  load_table(T, gT, bar, uses, status);
+  const Table& T = *gT;
   const long long N = P.N;
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c >= N) return;
@@ -354,33 +367,9 @@ __global__ void __launch_bounds__(kVjpThreads) vjp_kernel(Params P, const Table*
 #pragma unroll
   for (int e = 0; e < NB; ++e) lc[e] = lam[c * NB + e];
 
-  if (g_unew) {
-    // J^T lambda: the blocks (n, c) of column c, found in closed form as in
-    // spmv_grid_t_kernel, in the order of row c's columns
-    int ci, cj, ck;
-    cell_ijk(P, c, ci, cj, ck);
-    const bool hc[7] = {ck > 0, cj > 0, ci > 0, true, ci + 1 < P.nx, cj + 1 < P.ny, ck + 1 < P.nz};
-    const long long off[7] = {-P.nxy, -P.nx, -1, 0, 1, P.nx, P.nxy};
+  if (g_unew) {                          // J^T lambda
     double acc[NB];
-#pragma unroll
-    for (int v = 0; v < NB; ++v) acc[v] = 0.0;
-#pragma unroll
-    for (int t = 0; t < 7; ++t) {
-      if (!hc[t]) continue;
-      const long long n = c + off[t];
-      const int ni = ci + (t == 4) - (t == 2), nj = cj + (t == 5) - (t == 1), nk = ck + (t == 6) - (t == 0);
-      const bool hn[6] = {nk > 0, nj > 0, ni > 0, true, ni + 1 < P.nx, nj + 1 < P.ny};
-      int sn = 0;
-#pragma unroll
-      for (int u = 0; u < 6 - t; ++u) sn += hn[u];
-      const double* blk = val + (row_start_ijk(P, n, ni, nj, nk) + sn) * NB * NB;
-#pragma unroll
-      for (int e = 0; e < NB; ++e) {
-        const double l = lam[n * NB + e];
-#pragma unroll
-        for (int v = 0; v < NB; ++v) acc[v] = fma(blk[e * NB + v], l, acc[v]);
-      }
-    }
+    column_product<NB>(P, c, val, lam, acc);
 #pragma unroll
     for (int v = 0; v < NB; ++v) g_unew[v * N + c] = acc[v];
   }
@@ -396,18 +385,17 @@ __global__ void __launch_bounds__(kVjpThreads) vjp_kernel(Params P, const Table*
     double mo[3], m_p[3], m_sw[3], m_x[3];
     cell_masses<NB, true>(P, T, po, swo, xo, fo, 1.0, mo, m_p, m_sw, m_x);
     if (g_uold) {
-      double lph[NB];
-#pragma unroll
-      for (int e = 0; e < NB; ++e) lph[e] = lc[e] * ph;
-      double g[3] = {0.0, 0.0, 0.0};
+      const double w = neg(scale * ph);
+      double g[3];
 #pragma unroll
       for (int e = 0; e < NB; ++e) {
-        g[0] = fma(lph[e], m_p[e], g[0]);
-        g[1] = fma(lph[e], m_sw[e], g[1]);
-        g[2] = fma(lph[e], m_x[e], g[2]);
+        const double lw = lc[e] * w;
+        g[0] = e ? fma(lw, m_p[e], g[0]) : lw * m_p[e];
+        g[1] = e ? fma(lw, m_sw[e], g[1]) : lw * m_sw[e];
+        if (e) g[2] = e > 1 ? fma(lw, m_x[e], g[2]) : lw * m_x[e];    // the water's amount does not depend on X
       }
 #pragma unroll
-      for (int v = 0; v < NB; ++v) g_uold[v * N + c] = -scale * g[v];
+      for (int v = 0; v < NB; ++v) g_uold[v * N + c] = g[v];
     }
     if (g_phi) {
       double mn[3];
@@ -507,7 +495,7 @@ cudaError_t launch_spmv(const ocp_grid* g, const double* val, double alpha, cons
     return launch_pdl(spmv_grid_kernel<3>, gblocks, kSpmvThreads, 0, s, g->prm, (const int32_t*)g->d_row_ptr, val, alpha, x, beta, y, mode);
   }
   if (transpose) return launch_pdl(spmv_grid_t_kernel<2>, gblocks, kSpmvThreads, 0, s, g->prm, val, alpha, x, beta, y, mode);
-  if (bulk) return launch_pdl(spmv_bulk_kernel<2>, bblocks, kBulkRows, bulk_smem_bytes<2>(), s, g->prm, (const int32_t*)g->d_row_ptr, (long long)g->nnzb, val, alpha, x, beta, y, mode, g->d_status);
+  if (bulk) return launch_pdl(spmv_bulk_kernel<2>, bblocks, kBulkRows, bulk_smem_bytes<2>(), s, g->prm, (long long)g->nnzb, val, alpha, x, beta, y, mode, g->d_status);
   return launch_pdl(spmv_grid_kernel<2>, gblocks, kSpmvThreads, 0, s, g->prm, (const int32_t*)g->d_row_ptr, val, alpha, x, beta, y, mode);
 }
 
@@ -522,11 +510,11 @@ cudaError_t launch_vjp(const ocp_grid* g, const double* u_new, const int8_t* f_n
     return launch_pdl(vjp_kernel<3>, blocks, kVjpThreads, 0, s, P, (const Table*)g->d_table, u_new, f_new, u_old,
                       f_old, (const double*)g->d_phi, val, face_flux, (const double*)g->d_wlnk,
                       (const int32_t*)g->d_perf_of_cell, (const Perf*)g->d_perf, scale, lam, g_unew, g_uold, g_lnk,
-                      g_phi, g->d_status);
+                      g_phi);
   return launch_pdl(vjp_kernel<2>, blocks, kVjpThreads, 0, s, P, (const Table*)g->d_table, u_new, f_new, u_old,
                     f_old, (const double*)g->d_phi, val, face_flux, (const double*)g->d_wlnk,
                     (const int32_t*)g->d_perf_of_cell, (const Perf*)g->d_perf, scale, lam, g_unew, g_uold, g_lnk,
-                    g_phi, g->d_status);
+                    g_phi);
 }
 
 cudaError_t launch_well_rates(const ocp_grid* g, const double* u, const int8_t* flag, double* q,
