@@ -15,23 +15,23 @@
 // one's.  Applying D^-1 to the matrix once leaves 54 + 54 + 33 FMAs per cell
 // and iteration (3x3 blocks) where A x followed by D^-1 takes 177, and one
 // launch replaces the seven an iteration took.  Measured per iteration, both
-// at the same calls: 300 cells 45 -> 16 us, 100 000 cells 73 -> 46 us, 200 000
-// cells 118 -> 74 us, the scalar systems of IMPEC at 200 000 cells 50 -> 26 us;
-// the FP64 units' own time is 23 us at 100 000 cells.  The planes are read coalesced, each
-// thread its own entries; the vectors only their owner reads (r, r0, v, t, x,
-// the own parts of p and s) stay in shared memory where the range fits.  Only
-// p and s, which neighbours gather, go through L2.
+// at the same calls: 300 cells 45 -> 12 us, 100 000 cells 73 -> 45 us, 200 000
+// cells 118 -> 73 us, the scalar systems of IMPEC at 200 000 cells 50 -> 26 us;
+// the FP64 units' own time is 24 us at 100 000 cells.  The planes are read
+// coalesced, each thread its own entries; the vectors only their owner reads
+// (r, r0, v, t, x, the own parts of p and s) stay in shared memory where the
+// range fits.  Only p and s, which neighbours gather, go through L2.
 //
-// Grid barriers: every CTA stores the barrier's number in its slot of every
-// CTA's inbox and waits for the slots of its own, so no two CTAs poll the same
-// lines.  (With one set of slots that all CTAs polled, 152 CTAs kept its few
-// lines so busy that a barrier took 4.8 us, against 1.4 us among 8 CTAs; with
-// inboxes 2.5 us.)  A reduction stores the CTA's sums before its barrier, and
-// every CTA adds all CTAs' sums after it, in the same order, so that all get
-// the same bits.  The launch is cooperative (all CTAs are resident); the
-// waits are bounded.
+// Grid barriers and reductions: every CTA stores its partial sums with the
+// barrier's number, 16 bytes a value, in its slots of every CTA's inbox, waits
+// for the slots of its own inbox and adds them in the same order as every
+// other CTA, so that all get the same bits.  No two CTAs poll the same lines.
+// (With one set of slots that all CTAs polled, 152 CTAs kept its few lines so
+// busy that a barrier took 4.8 us, against 1.4 us among 8 CTAs; with inboxes
+// 2.5 us.)  The launch is cooperative (all CTAs are resident); the waits are
+// bounded.  Small systems run as one thread-block cluster instead, with the
+// hardware's barrier and sums through distributed shared memory.
 #include <cmath>
-#include <cstddef>
 
 #include "kernels.cuh"
 #include "ocp_internal.cuh"
@@ -44,17 +44,25 @@ constexpr int kMinRange = 128;         // unknowns of a CTA at least: one warp p
 constexpr int kMaxCtas = 256;
 constexpr int kVecs = 7;               // r, r0, p, v, s, t, x
 constexpr unsigned kSpin = 1u << 21;   // polls of one slot, above a second
-constexpr int kSmemVecBytes = 214 * 1024;
+constexpr int kSmemVecBytes = 213 * 1024;
+// The one-cluster launch takes systems of at most so many unknowns per CTA of
+// the largest cluster.  Per iteration, cluster / cooperative launch: 300 cells
+// (3x3) 12.2 / 15.6 us, 1260 13.5 / 14.9, 1728 15.1 / 15.7, 2400 16.8 / 16.7;
+// scalar 5400 cells 13.5 / 16.2, 9600 17.5 / 16.4.
+constexpr int kClusterRange = 384;
+constexpr int kClusterSmem = 120 * 1024;   // above half an SM's: the cluster's CTAs run on different SMs
 
-// Device data the grid keeps for its solves: the results; the CTAs' partial
-// sums, [barrier parity][value][CTA]; and an inbox of slots per CTA, [CTA]
-// [barrier parity][sender].  The barriers' numbers go on from one solve to the
-// next, so nothing is cleared in between.
+// Device data the grid keeps for its solves: the results, then an inbox of
+// slots per CTA, [CTA][barrier parity][value][sender].  The barriers' numbers
+// go on from one solve to the next, so nothing is cleared in between.
 struct SolveResult {
   double finished, iterations, rr, bb;
   unsigned long long epoch;
   double pad[3];
-  double sums[2][3][kMaxCtas];
+};
+struct alignas(16) Slot {
+  double v;
+  unsigned long long epoch;
 };
 
 struct SolveArgs {
@@ -73,17 +81,27 @@ struct SolveArgs {
   double rtol;
   int maxit;
   SolveResult* result;
-  unsigned long long* inbox;
+  Slot* inbox;
   unsigned long long epoch;            // number of the last barrier of earlier solves
   int* status;
 };
 
-__device__ __forceinline__ void slot_store(unsigned long long* p, unsigned long long epoch) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(epoch) : "memory");
+// A value and its barrier's number travel in one 16-byte relaxed access.
+__device__ __forceinline__ void slot_store(Slot* p, double v, unsigned long long epoch) {
+  asm volatile(
+      "{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p),
+      "l"(__double_as_longlong(v)), "l"(epoch)
+      : "memory");
 }
-__device__ __forceinline__ unsigned long long slot_load(const unsigned long long* p) {
+__device__ __forceinline__ unsigned long long slot_load(const Slot* p, double& v) {
+  long long a;
   unsigned long long epoch;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(epoch) : "l"(p) : "memory");
+  asm volatile(
+      "{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+      : "=l"(a), "=l"(epoch)
+      : "l"(p)
+      : "memory");
+  v = __longlong_as_double(a);
   return epoch;
 }
 __device__ __forceinline__ double load_plane(const double* p) {
@@ -347,27 +365,42 @@ __device__ __forceinline__ double well_part(const SolveArgs& A, int i, int ip, c
 
 // -------------------------------------------------------------- reductions
 struct Shared {
-  double red[3 * kSolveThreads];       // partial sums of the threads
+  double red[3 * kSolveThreads];       // partial sums of the threads, then of the CTAs
   double warp[3][4];
+  double cta[3];                       // the CTA's sums
+  double peers[2][3][kMaxClusterTiles];    // one-cluster launch: every CTA's sums, written by them
   double grid[3];                      // the grid's sums
   double out[4];
 };
 
 // A grid barrier that also sums NV values over the grid (NV = 0: only a
 // barrier), in two halves, so that a thread can work between them: grid_arrive
-// sends the CTA's sums, grid_wait collects the others'.  Warp 0 does both:
-// the CTA's writes before grid_arrive happen before its slot stores through
-// the CTA barrier and the warp's fence, and the fence after the polling and
-// the last CTA barrier order every thread's reads after it.  Slots and sums
-// alternate between two sets, since a CTA can enter the next barrier while
-// another still reads this one's, but not the one after.
+// sends the CTA's sums, grid_wait collects the others'.
+//
+// FENCE: the CTA's writes before it are visible to every CTA after it: they
+// happen before the slot stores, through the CTA barrier and the storing
+// threads' fences, and the fences after the polling and the last CTA barrier
+// order every thread's reads after it.  The reductions inside the iteration do
+// without (their fences took 1 us of 7): the sums travel in the slots
+// themselves, and the vectors are only exchanged across the fenced barriers --
+// p is published before one and read before the next, s likewise, so between
+// any CTA's reads of p (s) and the next writes of it lies the other's fenced
+// barrier.
+//
+// Slots alternate between two sets, since a CTA can enter the next barrier
+// while another still polls this one's slots, but not the one after.
 __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
-__device__ __forceinline__ unsigned long long* inbox_of(const SolveArgs& A, unsigned long long epoch, int cta) {
-  return A.inbox + ((long long)cta * 2 + (long long)(epoch & 1)) * A.ctas;
+__device__ __forceinline__ Slot* inbox_of(const SolveArgs& A, unsigned long long epoch, int cta, int q) {
+  return A.inbox + (((long long)cta * 2 + (long long)(epoch & 1)) * 3 + q) * A.ctas;
 }
 
-template <int NV>
+//
+// CLUSTER: the grid is one thread-block cluster (small systems, whose time is
+// barriers): the sums are stored into the CTAs' shared memory, and the
+// hardware's cluster barrier in its two halves takes the slots' place and
+// orders the vectors in global memory too.
+template <int NV, bool FENCE, bool CLUSTER>
 __device__ __forceinline__ void grid_arrive(const SolveArgs& A, Shared& sh, unsigned long long& epoch,
                                             const double (&part)[3]) {
   const int tid = threadIdx.x, T = blockDim.x, G = A.ctas;
@@ -402,43 +435,85 @@ __device__ __forceinline__ void grid_arrive(const SolveArgs& A, Shared& sh, unsi
       if (lane == 16) sh.warp[1][tid >> 5] = x;
       if (NV == 3 && lane == 8) sh.warp[2][tid >> 5] = x;
     }
-  }
-  __syncthreads();
-  if (tid < 32) {
+    __syncthreads();
     if (tid < NV) {
       const double* w = sh.warp[tid];
-      __stcg(&A.result->sums[epoch & 1][tid][blockIdx.x], ((w[0] + w[1]) + w[2]) + w[3]);
+      sh.cta[tid] = ((w[0] + w[1]) + w[2]) + w[3];
     }
-    __syncwarp();
-    fence_gpu();
-    for (int k = tid; k < G; k += 32) slot_store(inbox_of(A, epoch, k) + blockIdx.x, epoch);
+  }
+  if constexpr (CLUSTER) {
+    if constexpr (NV > 0) {
+      __syncthreads();
+      if (tid < NV * G) {
+        const int q = (tid >= G) + (tid >= 2 * G);
+        unsigned at;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                     : "=r"(at)
+                     : "r"((unsigned)__cvta_generic_to_shared(&sh.peers[epoch & 1][q][blockIdx.x])), "r"(tid - q * G));
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at), "d"(sh.cta[q]) : "memory");
+      }
+    }
+    if constexpr (NV == 0) __syncthreads();    // the CTA's own values are read between the halves
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    return;
+  }
+  __syncthreads();
+  constexpr int nv = NV > 0 ? NV : 1;
+  if (FENCE && tid < nv * G) fence_gpu();
+  for (int k = tid; k < nv * G; k += T) {
+    const int q = (k >= G) + (k >= 2 * G);
+    slot_store(inbox_of(A, epoch, k - q * G, q) + blockIdx.x, NV > 0 ? sh.cta[q] : 0.0, epoch);
   }
 }
 
 // With NV > 0 the sums are left in sh.grid for every thread.  Returns false
 // (in every thread) if a wait ran out.
-template <int NV>
+template <int NV, bool FENCE, bool CLUSTER>
 __device__ __forceinline__ bool grid_wait(const SolveArgs& A, Shared& sh, unsigned long long epoch) {
-  const int tid = threadIdx.x, G = A.ctas;
+  constexpr int nv = NV > 0 ? NV : 1, kPer = (nv * kMaxCtas + 127) / 128;    // at most so many slots a thread
+  const int tid = threadIdx.x, T = blockDim.x, G = A.ctas;
+  if constexpr (CLUSTER) {
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    if constexpr (NV > 0) {
+      const int q = tid >> 5, lane = tid & 31;
+      if (q < NV) {
+        double s = lane < G ? sh.peers[epoch & 1][q][lane] : 0.0;
+#pragma unroll
+        for (int o = kMaxClusterTiles / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) sh.grid[q] = s;
+      }
+      __syncthreads();
+    }
+    return true;
+  }
   bool ok = true;
-  if (tid < 32) {
-    const unsigned long long* in = inbox_of(A, epoch, blockIdx.x);
+  if (tid < nv * G) {
+    const Slot* in = inbox_of(A, epoch, blockIdx.x, 0);    // the values' slots are consecutive
+    double v[kPer];
     unsigned it = 0;
     for (bool all = false; !all;) {
-      all = tid >= G || slot_load(in + tid) == epoch;
-      if (G > 32) {                      // the others' loads in flight together
-        unsigned long long got[kMaxCtas / 32 - 1];
+      all = slot_load(in + tid, v[0]) == epoch;
+      if (nv * G > T) {                  // the others' loads in flight together
+        unsigned long long got[kPer];
 #pragma unroll
-        for (int j = 1; j < kMaxCtas / 32; ++j) got[j - 1] = tid + 32 * j < G ? slot_load(in + tid + 32 * j) : epoch;
+        for (int j = 1; j < kPer; ++j) got[j] = tid + j * T < nv * G ? slot_load(in + tid + j * T, v[j]) : epoch;
 #pragma unroll
-        for (int j = 1; j < kMaxCtas / 32; ++j) all = all && got[j - 1] == epoch;
+        for (int j = 1; j < kPer; ++j) all = all && got[j] == epoch;
       }
       if (!all && ++it == kSpin) {
         ok = false;
         break;
       }
     }
-    fence_gpu();
+    if constexpr (NV > 0) {
+      sh.red[tid] = v[0];
+      if (nv * G > T) {
+#pragma unroll
+        for (int j = 1; j < kPer; ++j)
+          if (tid + j * T < nv * G) sh.red[tid + j * T] = v[j];
+      }
+    }
+    if (FENCE) fence_gpu();
   }
   if (!__syncthreads_and(ok)) {
     if (tid == 0) atomicOr(A.status, kStatTimeout);
@@ -447,18 +522,8 @@ __device__ __forceinline__ bool grid_wait(const SolveArgs& A, Shared& sh, unsign
   if constexpr (NV > 0) {
     const int q = tid >> 5, lane = tid & 31;
     if (q < NV) {                        // one warp per value
-      const double* sums = A.result->sums[epoch & 1][q];
-      double s = lane < G ? __ldcg(sums + lane) : 0.0;
-      if (G > 32) {
-        double w[kMaxCtas / 32 - 1];
-#pragma unroll
-        for (int j = 1; j < kMaxCtas / 32; ++j) w[j - 1] = lane + 32 * j < G ? __ldcg(sums + lane + 32 * j) : 0.0;
-#pragma unroll
-        for (int j = 1; j < kMaxCtas / 32; ++j) {
-          if (32 * j >= G) break;
-          s += w[j - 1];
-        }
-      }
+      double s = lane < G ? sh.red[q * G + lane] : 0.0;
+      for (int k = lane + 32; k < G; k += 32) s += sh.red[q * G + k];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
       if (lane == 0) sh.grid[q] = s;
@@ -478,7 +543,7 @@ __device__ __forceinline__ bool grid_wait(const SolveArgs& A, Shared& sh, unsign
 // and r . r, which only the loop's test needs, come with r0 . v.  The test
 // then costs a solve half an iteration, a third reduction 5 us of the 45 of
 // every iteration at 100 000 cells.
-template <int NB, bool WELLS, bool PLANES>
+template <int NB, bool WELLS, bool PLANES, bool CLUSTER>
 __global__ void __launch_bounds__(kSolveThreads, 1) solve_kernel(const __grid_constant__ SolveArgs A) {
   extern __shared__ double dyn[];
   __shared__ Shared sh;
@@ -494,48 +559,52 @@ __global__ void __launch_bounds__(kSolveThreads, 1) solve_kernel(const __grid_co
   const bool sm_p = A.smem_vecs > 2, sm_s = A.smem_vecs > 3;
   unsigned long long epoch = A.epoch;
   double part[3] = {0.0, 0.0, 0.0};
+  // no CTA's shared memory is written before the CTA runs
+  if constexpr (CLUSTER) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
   // first parts of M src that need only the CTA's own values (`mine`), to out
   auto apply_near = [&](const double* mine, double* out) {
-    if (!PLANES) return;
-    for (int l = tid; l < len; l += T) {
-      const RowAt w = row_at<NB>(A.P, base + l);
-      if (near_row<NB>(A.P, w, base, len)) out[l] = row_xy<NB>(A, w, base + l, mine + (w.c * NB - base), mine[l]);
+    if constexpr (PLANES) {
+      for (int l = tid; l < len; l += T) {
+        const RowAt w = row_at<NB>(A.P, base + l);
+        if (near_row<NB>(A.P, w, base, len)) out[l] = row_xy<NB>(A, w, base + l, mine + (w.c * NB - base), mine[l]);
+      }
     }
   };
-  // element l of M src (whole warps call it); `begun`: where apply_near left its part, or null
-  auto apply = [&](int l, const double* src, const double* begun) {
-    const bool live = l < len;
-    const int i = base + (live ? l : len - 1);
-    double acc;
-    if (PLANES) {
-      const RowAt w = row_at<NB>(A.P, i);
-      const double* xc = src + (long long)w.c * NB;
-      if (begun && live && near_row<NB>(A.P, w, base, len)) acc = begun[l];
-      else acc = row_xy<NB>(A, w, i, xc, src[i]);
-      acc = row_z<NB>(A, w, i, xc, acc);
-    } else {
-      acc = row_product_unscaled<NB>(A, i, src);
+  // use(l, (M src)_l) for every element of this thread; `begun`: where
+  // apply_near left its parts, or null
+  auto apply = [&](const double* src, const double* begun, auto&& use) {
+    for (int l0 = tid & ~31; l0 < len; l0 += T) {    // whole warps
+      const int l = l0 + (tid & 31);
+      const bool live = l < len;
+      const int i = base + (live ? l : len - 1);
+      double acc;
+      if (PLANES) {
+        const RowAt w = row_at<NB>(A.P, i);
+        const double* xc = src + (long long)w.c * NB;
+        if (begun && live && near_row<NB>(A.P, w, base, len)) acc = begun[l];
+        else acc = row_xy<NB>(A, w, i, xc, src[i]);
+        acc = row_z<NB>(A, w, i, xc, acc);
+      } else {
+        acc = row_product_unscaled<NB>(A, i, src);
+      }
+      if (WELLS) acc = well_part<NB>(A, i, live ? A.perf_of_cell[i / NB] : -1, src, acc);
+      if (live) use(l, acc);
     }
-    if (WELLS) acc = well_part<NB>(A, i, live ? A.perf_of_cell[i / NB] : -1, src, acc);
-    return acc;
   };
   // y = D^-1 b stands in vec[0]; r0 = p = r = y - M x
-  for (int l0 = tid & ~31; l0 < len; l0 += T) {
-    const int l = l0 + (tid & 31);
-    const double m = apply(l, A.vec[6], nullptr);
-    if (l < len) {
-      const double y = A.vec[0][base + l], ri = y - m;
-      r[l] = ri;
-      r0[l] = ri;
-      p[l] = ri;
-      if (sm_p) pub_p[l] = ri;
-      if (A.smem_vecs > 6) x[l] = A.vec[6][base + l];
-      part[0] = fma(y, y, part[0]);
-      part[1] = fma(ri, ri, part[1]);
-    }
-  }
-  grid_arrive<2>(A, sh, epoch, part);
-  if (!grid_wait<2>(A, sh, epoch)) return;
+  apply(A.vec[6], nullptr, [&](int l, double m) {
+    const double y = A.vec[0][base + l], ri = y - m;
+    r[l] = ri;
+    r0[l] = ri;
+    p[l] = ri;
+    if (sm_p) pub_p[l] = ri;
+    if (A.smem_vecs > 6) x[l] = A.vec[6][base + l];
+    part[0] = fma(y, y, part[0]);
+    part[1] = fma(ri, ri, part[1]);
+  });
+  if constexpr (CLUSTER) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  grid_arrive<2, true, CLUSTER>(A, sh, epoch, part);
+  if (!grid_wait<2, true, CLUSTER>(A, sh, epoch)) return;
   const double bb = sh.grid[0];
   double rr = sh.grid[1], rho = rr, alpha = 1.0, omega = 1.0, beta = 0.0;
   const double bnorm = sqrt(bb), target = A.rtol * (bnorm > 0.0 ? bnorm : 1.0);
@@ -546,16 +615,12 @@ __global__ void __launch_bounds__(kSolveThreads, 1) solve_kernel(const __grid_co
   apply_near(p, v);
   while (go) {
     // v = M p, then alpha and the test on r . r
-    for (int l0 = tid & ~31; l0 < len; l0 += T) {
-      const int l = l0 + (tid & 31);
-      const double vi = apply(l, A.vec[2], v);
-      if (l < len) {
-        v[l] = vi;
-        part[0] = fma(r0[l], vi, part[0]);
-      }
-    }
-    grid_arrive<3>(A, sh, epoch, part);
-    if (!grid_wait<3>(A, sh, epoch)) return;
+    apply(A.vec[2], v, [&](int l, double vi) {
+      v[l] = vi;
+      part[0] = fma(r0[l], vi, part[0]);
+    });
+    grid_arrive<3, false, CLUSTER>(A, sh, epoch, part);
+    if (!grid_wait<3, false, CLUSTER>(A, sh, epoch)) return;
     if (iter > 0) rho = sh.grid[2];
     if (tid == 0) {
       const double a = sh.grid[0];
@@ -577,27 +642,23 @@ __global__ void __launch_bounds__(kSolveThreads, 1) solve_kernel(const __grid_co
       s[l] = si;
       if (sm_s) pub_s[l] = si;
     }
-    grid_arrive<0>(A, sh, epoch, part);
+    grid_arrive<0, true, CLUSTER>(A, sh, epoch, part);
     apply_near(s, t);
-    if (!grid_wait<0>(A, sh, epoch)) return;
+    if (!grid_wait<0, true, CLUSTER>(A, sh, epoch)) return;
     // t = M s, then omega and rho
     part[0] = part[1] = part[2] = 0.0;
-    for (int l0 = tid & ~31; l0 < len; l0 += T) {
-      const int l = l0 + (tid & 31);
-      const double ti = apply(l, A.vec[3], t);
-      if (l < len) {
-        t[l] = ti;
-        part[0] = fma(ti, s[l], part[0]);
-        part[1] = fma(ti, ti, part[1]);
-        part[2] = fma(r0[l], ti, part[2]);
-      }
-    }
-    grid_arrive<3>(A, sh, epoch, part);
+    apply(A.vec[3], t, [&](int l, double ti) {
+      t[l] = ti;
+      part[0] = fma(ti, s[l], part[0]);
+      part[1] = fma(ti, ti, part[1]);
+      part[2] = fma(r0[l], ti, part[2]);
+    });
+    grid_arrive<3, false, CLUSTER>(A, sh, epoch, part);
     // x += alpha p + omega s, each term while a barrier is on its way
     for (int l = tid; l < len; l += T) x[l] = fma(alpha, p[l], x[l]);
     double ratio = 0.0;
     if (tid == 0) ratio = alpha / rho;
-    if (!grid_wait<3>(A, sh, epoch)) return;
+    if (!grid_wait<3, false, CLUSTER>(A, sh, epoch)) return;
     if (tid == 0) {
       const double ts = sh.grid[0], tt = sh.grid[1], r0t = sh.grid[2];
       const double om = tt == 0.0 ? 0.0 : ts / tt;    // t = 0: s = 0 and x is already exact
@@ -621,10 +682,10 @@ __global__ void __launch_bounds__(kSolveThreads, 1) solve_kernel(const __grid_co
       if (sm_p) pub_p[l] = pi;
     }
     ++iter;
-    grid_arrive<0>(A, sh, epoch, part);
+    grid_arrive<0, true, CLUSTER>(A, sh, epoch, part);
     for (int l = tid; l < len; l += T) x[l] = fma(omega, s[l], x[l]);
     apply_near(p, v);
-    if (!grid_wait<0>(A, sh, epoch)) return;
+    if (!grid_wait<0, true, CLUSTER>(A, sh, epoch)) return;
   }
   if (A.smem_vecs > 6)
     for (int l = tid; l < len; l += T) A.vec[6][base + l] = x[l];
@@ -637,11 +698,10 @@ __global__ void __launch_bounds__(kSolveThreads, 1) solve_kernel(const __grid_co
   }
 }
 
-template <int NB>
-const void* solve_function(bool wells, bool planes) {
-  if constexpr (NB > 1)                  // scalar systems come without well unknowns
-    if (wells) return planes ? (const void*)solve_kernel<NB, true, true> : (const void*)solve_kernel<NB, true, false>;
-  return planes ? (const void*)solve_kernel<NB, false, true> : (const void*)solve_kernel<NB, false, false>;
+template <int NB, bool WELLS>
+const void* solve_function(bool planes, bool cluster) {
+  if (cluster) return (const void*)solve_kernel<NB, WELLS, true, true>;
+  return planes ? (const void*)solve_kernel<NB, WELLS, true, false> : (const void*)solve_kernel<NB, WELLS, false, false>;
 }
 
 }  // namespace
@@ -666,7 +726,7 @@ ocp_status bicgstab_run(ocp_grid* g, const double* val, const WellSchur* ws, con
   const long long N = g->prm.N, n = nb * N;
   cudaError_t e = cudaSuccess;
   const int sms = g->sms < kMaxCtas ? g->sms : kMaxCtas;
-  const size_t sync_bytes = sizeof(SolveResult) + sizeof(unsigned long long) * 2 * (size_t)sms * sms;
+  const size_t sync_bytes = sizeof(SolveResult) + sizeof(Slot) * 6 * (size_t)sms * sms;
   if (!g->d_solve_sync) {
     e = cudaMalloc((void**)&g->d_solve_sync, sync_bytes);
     if (e != cudaSuccess) {
@@ -694,8 +754,10 @@ ocp_status bicgstab_run(ocp_grid* g, const double* val, const WellSchur* ws, con
   SolveArgs A{};
   A.P = g->prm;
   A.n = (int)n;
+  const int most = g->max_cluster < kMaxClusterTiles ? g->max_cluster : kMaxClusterTiles;
+  const bool cluster = planes && most > 0 && n <= (long long)most * kClusterRange;
   long long ctas = (n + kMinRange - 1) / kMinRange;
-  if (ctas > sms) ctas = sms;
+  if (ctas > (cluster ? most : sms)) ctas = cluster ? most : sms;
   A.range = (int)(((n + ctas - 1) / ctas + 31) / 32 * 32);
   A.ctas = (int)((n + A.range - 1) / A.range);
   const int threads = A.range < 128 ? 128 : (A.range < kSolveThreads ? A.range : kSolveThreads);
@@ -716,27 +778,45 @@ ocp_status bicgstab_run(ocp_grid* g, const double* val, const WellSchur* ws, con
   A.rtol = rtol;
   A.maxit = maxit;
   A.result = (SolveResult*)g->d_solve_sync;
-  A.inbox = (unsigned long long*)(A.result + 1);
+  A.inbox = (Slot*)(A.result + 1);
   A.epoch = g->solve_epoch;
   A.status = g->d_status;
   const WellSchur wsv = ws ? *ws : WellSchur{nullptr, nullptr, nullptr};
-  if (e == cudaSuccess) e = cudaMemsetAsync(g->d_solve_sync, 0, offsetof(SolveResult, sums), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(g->d_solve_sync, 0, sizeof(SolveResult), s);
   const unsigned blocks = (unsigned)((n + 255) / 256);
   double* dinv = planes ? nullptr : work + 8 * n;
   auto scale = nb == 3 ? scale_kernel<3> : (nb == 2 ? scale_kernel<2> : scale_kernel<1>);
   if (e == cudaSuccess)
     e = launch_pdl(scale, blocks, 256, 0, s, g->prm, (int)n, val, A.trans, (const int32_t*)g->d_perf_of_cell,
                    (const Perf*)g->d_perf, wsv, b, planes, dinv, A.vec[0], wb, g->d_status);
-  const void* fn = nb == 3   ? solve_function<3>(ws != nullptr, planes != nullptr)
-                   : nb == 2 ? solve_function<2>(ws != nullptr, planes != nullptr)
-                             : solve_function<1>(ws != nullptr, planes != nullptr);
-  const int smem = 8 * A.smem_vecs * A.range;
+  const bool pl = planes != nullptr;
+  const void* fn = nb == 3   ? (ws ? solve_function<3, true>(pl, cluster) : solve_function<3, false>(pl, cluster))
+                   : nb == 2 ? (ws ? solve_function<2, true>(pl, cluster) : solve_function<2, false>(pl, cluster))
+                             : solve_function<1, false>(pl, cluster);     // scalar systems have no well unknowns
+  int smem = 8 * A.smem_vecs * A.range;
+  if (cluster && smem < kClusterSmem) smem = kClusterSmem;
   if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemVecBytes);
+  if (e == cudaSuccess && cluster) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   void* args[] = {&A};
-  if (e == cudaSuccess)
-    e = cudaLaunchCooperativeKernel(fn, dim3((unsigned)A.ctas), dim3((unsigned)threads), args, (size_t)smem, s);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)A.ctas);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  if (cluster) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)A.ctas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  } else {
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (e == cudaSuccess) e = cudaLaunchKernelExC(&cfg, fn, args);
   SolveResult h{};
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, g->d_solve_sync, offsetof(SolveResult, sums), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, g->d_solve_sync, sizeof(h), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   g->solve_epoch = e == cudaSuccess && h.finished != 0.0 ? h.epoch : 0;
   if (e != cudaSuccess) return report(OCP_ERR_CUDA, "ocp_bicgstab: %s", cudaGetErrorString(e));

@@ -1,8 +1,9 @@
 """The persistent BiCGSTAB on the GPU against dense solves.
 
 Sizes at the edges of its work split (an unknown per thread, 32-unknown
-chunks, CTAs of at least 128 unknowns, ranges that do not divide evenly),
-grids without one or two directions, both orientations, every block size,
+chunks, CTAs of at least 128 unknowns, ranges that do not divide evenly, the
+largest system of the one-cluster launch and the smallest above it), grids
+without one or two directions, both orientations, every block size,
 and the path without the scaled copy of the matrix.
 """
 import numpy as np
@@ -53,7 +54,7 @@ def _scaled_residual(A, x, b, nb):
 @pytest.mark.parametrize("transpose", [False, True])
 @pytest.mark.parametrize("nb", [1, 2, 3])
 @pytest.mark.parametrize("dims", [(1, 1, 1), (5, 1, 1), (1, 3, 1), (1, 1, 11), (7, 6, 1), (1, 9, 5), (4, 1, 8),
-                                  (8, 8, 2), (11, 4, 4), (9, 8, 7), (17, 13, 3)])
+                                  (8, 8, 2), (11, 4, 4), (9, 8, 7), (17, 13, 3), (16, 16, 8), (41, 5, 10)])
 def test_solves_random_block_systems(dims, nb, transpose):
     need_gpu()
     from paper_2406_10862_gb300 import ocp as O
