@@ -756,9 +756,15 @@ __device__ __forceinline__ void cell_masses(const Params& P, const Table& T, dou
 }
 
 // ---------------------------------------------------------------- face flux
-// Sign flip without an FP64 instruction.
+// Sign flip without an FP64 instruction: for values that are stored or
+// selected.  The compiler knows a flipped sign bit for a negation in any
+// C++ form and adds zero to it on the FP64 pipe; out of its sight it is one
+// integer instruction.  (The negated operand of a sum or product is free:
+// there, plain -x.)
 __device__ __forceinline__ double neg(double x) {
-  return __longlong_as_double(__double_as_longlong(x) ^ (long long)0x8000000000000000ULL);
+  int hi = __double2hiint(x);
+  asm("xor.b32 %0, %0, 0x80000000;" : "+r"(hi));
+  return __hiloint2double(hi, __double2loint(x));
 }
 
 // One phase across one face: F = T lambda_up dphi with dphi = (pa_i - pa_j)
@@ -802,7 +808,7 @@ __device__ __forceinline__ void phase_flux(double T, double hz, double pa_i, dou
   if (LSW) usw = Td * sel(up, l_sw_i, l_sw_j);
   if (PSW) {
     di[1] = fma(Tl, dpa_i, sel(up, usw, 0.0));
-    dj[1] = fma(neg(Tl), dpa_j, sel(up, 0.0, usw));
+    dj[1] = fma(-Tl, dpa_j, sel(up, 0.0, usw));
   } else {
     di[1] = sel(up, usw, 0.0);
     dj[1] = sel(up, 0.0, usw);
@@ -813,13 +819,13 @@ __device__ __forceinline__ void phase_flux(double T, double hz, double pa_i, dou
   dj[2] = sel(up, 0.0, ux);
   if (PX) {
     di[2] = fma(Tl, dpa_i, di[2]);
-    dj[2] = fma(Tl, neg(dpa_j), dj[2]);
+    dj[2] = fma(-Tl, dpa_j, dj[2]);
   } else if (GRAV && RX) {
     // saturated oil: the densities do not depend on X, and adding the zero
     // products changes nothing (where that holds for the whole warp)
     if (__any_sync(__activemask(), nonzero(rho_x_i) || nonzero(rho_x_j))) {
-      di[2] = fma(Tl, neg(rho_x_i * hz), di[2]);
-      dj[2] = fma(Tl, neg(rho_x_j * hz), dj[2]);
+      di[2] = fma(-Tl, rho_x_i * hz, di[2]);
+      dj[2] = fma(-Tl, rho_x_j * hz, dj[2]);
     }
   }
 }
