@@ -386,6 +386,17 @@ __device__ __forceinline__ bool nonzero(double x) {
   return ((unsigned)__double2loint(x) | ((unsigned)__double2hiint(x) & 0x7fffffffu)) != 0u;
 }
 
+// Sign flip without an FP64 instruction: for values that are stored or
+// selected.  The compiler knows a flipped sign bit for a negation in any
+// C++ form and adds zero to it on the FP64 pipe; out of its sight it is one
+// integer instruction.  (The negated operand of a sum or product is free:
+// there, plain -x.)
+__device__ __forceinline__ double neg(double x) {
+  int hi = __double2hiint(x);
+  asm("xor.b32 %0, %0, 0x80000000;" : "+r"(hi));
+  return __hiloint2double(hi, __double2loint(x));
+}
+
 // Largest k <= nrow-2 with key[k] <= xk (binary search on integer keys).
 __device__ __forceinline__ int segment(const long long* key, int nrow, long long xk) {
   int lo = 0, hi = nrow - 2;
@@ -508,36 +519,38 @@ __device__ __forceinline__ void pvt(const Params& P, const Table& T, double p, d
 // gas (so that the components can be split between warps).  SAT: the caller
 // knows the oil to be saturated (b_o and R_s do not depend on X = S_g); the
 // terms that are zero then are left out, the others are the same bits.
+// The amounts per unit saturation (phi b and its p-derivative) come first:
+// every derivative then is a product with them, 25 FP64 instructions with
+// three phases where one product after the other took 31.
 template <int NB, bool DERIV, int PART = 2, bool SAT = false>
 __device__ __forceinline__ void masses(const Params& P, const Pvt& f, double p, double sw, double phi_ref,
                                        double* m, double* m_p, double* m_sw, double* m_x) {
-  const double phi = phi_ref * fma(P.cr, p - P.p_ref, 1.0);
+  const double phi_p = phi_ref * P.cr;
+  const double phi = fma(phi_p, p - P.p_ref, phi_ref);
   const double so = (NB == 3) ? (1.0 - sw - f.sg) : (1.0 - sw);
-  const double sob = so * f.bo;
+  const double O = phi * f.bo, mo = so * O;
+  const double O_p = fma(phi_p, f.bo, phi * f.bo_p), mo_p = so * O_p;
+  const double mo_x = SAT ? neg(O) : fma(-f.sg_x, O, so * (phi * f.bo_x));
   if (PART != 1) {
-    m[0] = phi * sw * f.bw;
-    m[1] = phi * sob;
-  }
-  if (PART != 0 && NB == 3) m[2] = phi * fma(f.sg, f.bg, f.rs * sob);
-  if (DERIV) {
-    const double phi_p = phi_ref * P.cr;
-    const double so_x = -f.sg_x;
-    if (PART != 1) {
-      m_p[0] = fma(phi_p * sw, f.bw, phi * sw * f.bw_p);
-      m_sw[0] = phi * f.bw;
+    const double W = phi * f.bw;
+    m[0] = sw * W;
+    m[1] = mo;
+    if (DERIV) {
+      m_p[0] = sw * fma(phi_p, f.bw, phi * f.bw_p);
+      m_sw[0] = W;
       m_x[0] = 0.0;
-      m_p[1] = fma(phi_p, sob, phi * so * f.bo_p);
-      m_sw[1] = -phi * f.bo;
-      m_x[1] = SAT ? m_sw[1] : phi * fma(so_x, f.bo, so * f.bo_x);
+      m_p[1] = mo_p;
+      m_sw[1] = neg(O);
+      m_x[1] = mo_x;
     }
-    if (PART != 0 && NB == 3) {
-      const double G = fma(f.sg, f.bg, f.rs * sob);
-      const double G_p = fma(f.sg, f.bg_p, fma(f.rs_p, sob, f.rs * so * f.bo_p));
-      const double G_x = SAT ? __dadd_rn(f.bg, -__dmul_rn(f.rs, f.bo))
-                             : fma(f.sg_x, f.bg, fma(f.rs_x, sob, f.rs * fma(so_x, f.bo, so * f.bo_x)));
-      m_p[2] = fma(phi_p, G, phi * G_p);
-      m_sw[2] = -phi * f.rs * f.bo;
-      m_x[2] = phi * G_x;
+  }
+  if (PART != 0 && NB == 3) {
+    const double G = phi * f.bg, rso = f.rs * so;
+    m[2] = fma(rso, O, f.sg * G);
+    if (DERIV) {
+      m_p[2] = fma(rso, O_p, fma(f.rs_p, mo, f.sg * fma(phi_p, f.bg, phi * f.bg_p)));
+      m_sw[2] = -f.rs * O;
+      m_x[2] = SAT ? __dadd_rn(G, m_sw[2]) : fma(f.sg_x, G, fma(f.rs_x, mo, f.rs * mo_x));
     }
   }
 }
@@ -557,7 +570,7 @@ struct Kr {
 // combines them (so that the two sides can also run in different warps).
 struct KrSide {
   double s, s_d;               // clamped normalised S_w or S_g and its slope
-  double po, dpo, so_d;        // (s_ow or s_og)^n; its derivative in S_w or S_g is dpo so_d
+  double po, dpo, so_d;        // (s_ow or s_og)^n; its derivative in S_w or S_g is -dpo so_d
   double kr, kr_d;             // k_rw or k_rg and its derivative in S_w or S_g
 };
 // kr_d = kr_max (d s^n) (slope) in one product for exponent 2: the constants
@@ -565,7 +578,7 @@ struct KrSide {
 __device__ __forceinline__ void rel_perm_w(const Params& P, double sw, KrSide& w) {
   double s_w = (sw - P.swc) * P.inv_w, s_w_d = P.inv_w, s_w_k = P.krw2;
   clamp01(s_w, s_w_d, s_w_k);
-  double s_ow = (1.0 - sw - P.sorw) * P.inv_w, s_ow_d = -P.inv_w, s_ow_2 = -P.inv_w2;
+  double s_ow = (1.0 - sw - P.sorw) * P.inv_w, s_ow_d = P.inv_w, s_ow_2 = P.inv_w2;
   clamp01(s_ow, s_ow_d, s_ow_2);
   double pw_;
   if (P.sq_w) {
@@ -583,7 +596,7 @@ __device__ __forceinline__ void rel_perm_w(const Params& P, double sw, KrSide& w
 __device__ __forceinline__ void rel_perm_g(const Params& P, double sg, KrSide& g) {
   double s_g = (sg - P.sgc) * P.inv_g, s_g_d = P.inv_g, s_g_k = P.krg2;
   clamp01(s_g, s_g_d, s_g_k);
-  double s_og = (1.0 - sg - P.swc - P.sorg) * P.inv_og, s_og_d = -P.inv_og, s_og_2 = -P.inv_og2;
+  double s_og = (1.0 - sg - P.swc - P.sorg) * P.inv_og, s_og_d = P.inv_og, s_og_2 = P.inv_og2;
   clamp01(s_og, s_og_d, s_og_2);
   double pg_;
   if (P.sq_g) {
@@ -612,16 +625,16 @@ __device__ __forceinline__ void rel_perm_combine(const Params& P, const KrSide& 
     s_g_d = g.s_d;
     // k_ro = kc [(k_row/kc + k_rw)(k_rog/kc + k_rg) - (k_rw + k_rg)], k_row/kc = s_ow^n
     const double A = __dadd_rn(w.po, w.kr);
-    const double A_sw = fma(w.dpo, w.so_d, w.kr_d);
+    const double A_sw = fma(-w.dpo, w.so_d, w.kr_d);
     const double B = __dadd_rn(g.po, krg);
-    const double B_sg = fma(g.dpo, g.so_d, krg_sg);
+    const double B_sg = fma(-g.dpo, g.so_d, krg_sg);
     kro = P.kc * fma(A, B, -__dadd_rn(w.kr, krg));
     kro_sw = P.kc * fma(A_sw, B, -w.kr_d);
     kro_sg = P.kc * fma(A, B_sg, -krg_sg);
     if (!nonneg(kro)) { kro = 0.0; kro_sw = 0.0; kro_sg = 0.0; }
   } else {
     kro = P.kc * w.po;
-    kro_sw = P.kc * w.dpo * w.so_d;
+    kro_sw = -P.kc * w.dpo * w.so_d;
   }
   const bool gx = (NB == 3) && (flag == 0);
   k.krw = w.kr;
@@ -683,9 +696,9 @@ __device__ __forceinline__ void dens_mob(const Params& P, const Pvt& f, const Kr
     }
   }
   if (!O) return;
-  const double ro0 = fma(f.rs, P.cg, P.rho_osc);
+  const double ro0 = (NB == 3) ? fma(f.rs, P.cg, P.rho_osc) : P.rho_osc;
   q.ro = ro0 * f.bo;
-  q.ro_p = fma(P.cg * f.rs_p, f.bo, ro0 * f.bo_p);
+  q.ro_p = (NB == 3) ? fma(P.cg * f.rs_p, f.bo, ro0 * f.bo_p) : ro0 * f.bo_p;
   const double bmo = f.bo * f.imo;
   const double bmo_p = fma(f.bo_p, f.imo, f.bo * f.imo_p);
   q.lo = k.kro * bmo;
@@ -756,17 +769,6 @@ __device__ __forceinline__ void cell_masses(const Params& P, const Table& T, dou
 }
 
 // ---------------------------------------------------------------- face flux
-// Sign flip without an FP64 instruction: for values that are stored or
-// selected.  The compiler knows a flipped sign bit for a negation in any
-// C++ form and adds zero to it on the FP64 pipe; out of its sight it is one
-// integer instruction.  (The negated operand of a sum or product is free:
-// there, plain -x.)
-__device__ __forceinline__ double neg(double x) {
-  int hi = __double2hiint(x);
-  asm("xor.b32 %0, %0, 0x80000000;" : "+r"(hi));
-  return __hiloint2double(hi, __double2loint(x));
-}
-
 // One phase across one face: F = T lambda_up dphi with dphi = (pa_i - pa_j)
 // - gbar (z_i - z_j), gbar = g (rho_i + rho_j) / 2, and its derivatives in
 // the unknowns (p, S_w, X) of both cells.  `hz` = g (z_i - z_j) / 2; on
