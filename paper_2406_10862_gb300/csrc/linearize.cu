@@ -6,17 +6,18 @@
 //                    (ACCU) and well (AllWells) terms of every cell;
 //   face_kernel      the upwinded two-point flux of every face, computed
 //                    exactly once (BulkConn).  The thread of cell c handles
-//                    its +x, +y, +z faces: it writes the two off-diagonal
-//                    blocks of each face straight into the Jacobian, adds the
-//                    face to its own residual and diagonal block, and hands
-//                    the + neighbour its share (flux and diagonal block);
+//                    its +x, +y, +z faces: the two off-diagonal blocks of
+//                    each face go into the Jacobian (a warp's blocks together,
+//                    through shared memory), the face is added to the cell's
+//                    own residual and diagonal block, and the + neighbour is
+//                    handed its share (flux and diagonal block);
 //   assemble_kernel  every cell subtracts the shares handed to it and writes
 //                    its residual and diagonal block.
 // No atomics: every output entry has one writer and a fixed summation order
 // (own terms, +x, +y, +z, then -z, -y, -x), independent of the launch shape.
 // On GB300 the FP64 pipe, not HBM, bounds these kernels, so each face is
-// computed once and results travel through (coalesced, variable-major)
-// scratch rather than being recomputed.
+// computed once and results travel through (coalesced) scratch rather than
+// being recomputed.
 //
 // The outputs (Jacobian blocks, residual, face fluxes) are written with
 // streaming stores (evict-first), so that they do not push out of L2 the
@@ -44,9 +45,9 @@ namespace {
 // third line).
 constexpr int kQ = 25;      // CellQ fields            0 .. 24
 constexpr int kSelf = 25;   // own residual (3) + diagonal (9)   25 .. 36
-constexpr int kPart = 37;   // after the +faces                  37 .. 48
-constexpr int kInc = 49;    // shares handed over, 3 x (F 3 + dj 9)   49 .. 84
-constexpr int kFields = 85;
+constexpr int kPart = 25;   // the same after the + faces, in their place
+constexpr int kInc = 37;    // shares handed over, 3 x (F 3 + dj 9)   37 .. 72
+constexpr int kFields = 73;
 // A cell's scratch: field f is at cell_scratch(scr, c)[32 * f].
 __device__ __forceinline__ double* cell_scratch(double* scr, long long c) {
   return scr + ((c >> 5) * (32 * kFields) + (c & 31));
@@ -204,7 +205,6 @@ __device__ __forceinline__ void cell_body(const ModelArgs& M, const Table& T, lo
 template <int NB, bool COH>
 __device__ __forceinline__ void face_part(const ModelArgs& M, long long c, bool live, WarpStage<NB>& st,
                                           double (&r)[NB], double (&dg)[NB][NB]) {
-  constexpr int B2 = NB * NB;
   const Params& P = M.P;
   const long long N = P.N;
   double* __restrict__ val = M.val;
@@ -227,10 +227,14 @@ __device__ __forceinline__ void face_part(const ModelArgs& M, long long c, bool 
   }
   const long long row0 = row_start_ijk(P, c, i, j, k);   // the row pointers in closed form: no loads
   int slot = (int)hm[0] + (int)hm[1] + (int)hm[2] + 1;   // first + block of this row
-#pragma unroll 1
+  // unrolled: the direction is a constant in each copy (full linearisation of
+  // 30 000 and 400 000 cells 32.6 -> 31.5 and 288 -> 281 us); the ordered
+  // launch's one kernel, which also holds the other stages, would spill
+#pragma unroll (COH ? 1 : 3)
   for (int d = 0; d < 3; ++d) {
     FaceOut<NB> o;
-    double blk[NB][NB], *base = nullptr, *nbase = nullptr;
+    double blk[NB][NB];
+    BlockAt<NB> at, nat;
     if (hp[d]) {
       const long long n = c + stride[d];
       double* sn = cell_scratch(M.scr, n);
@@ -241,10 +245,10 @@ __device__ __forceinline__ void face_part(const ModelArgs& M, long long c, bool 
       else face_terms<NB, false>(T, 0.0, a, b, o);
       // this row: flux out, diagonal, and the block of the + neighbour; the
       // + neighbour's row: its share, and its block of this cell
-      base = val + (row0 + slot) * B2;
+      at.set(val, row0 + slot);
       ++slot;
       const int slot_n = (d == 0) ? ((int)hm[2] + (int)hm[1]) : (d == 1 ? (int)hm[2] : 0);
-      nbase = val + (row_start_ijk(P, n, i + (d == 0), j + (d == 1), k + (d == 2)) + slot_n) * B2;
+      nat.set(val, row_start_ijk(P, n, i + (d == 0), j + (d == 1), k + (d == 2)) + slot_n);
       sn += 32 * (kInc + 12 * d);
 #pragma unroll
       for (int e = 0; e < NB; ++e) {
@@ -264,12 +268,12 @@ __device__ __forceinline__ void face_part(const ModelArgs& M, long long c, bool 
       for (int e = 0; e < NB; ++e) face_flux[(d * NB + e) * N + c] = 0.0;
     }
     if (!__any_sync(0xffffffffu, hp[d])) continue;
-    store_blocks<NB>(st, blk, base);
+    store_blocks<NB>(st, blk, val, at);
 #pragma unroll
     for (int e = 0; e < NB; ++e)
 #pragma unroll
       for (int v = 0; v < NB; ++v) blk[e][v] = neg(o.di[e][v]);
-    store_blocks<NB>(st, blk, nbase);
+    store_blocks<NB>(st, blk, val, nat);
   }
 }
 
@@ -310,12 +314,13 @@ __device__ __forceinline__ void assemble_rows(const ModelArgs& M, long long c, b
         if (!face_zero<NB>(e, v)) dg[e][v] -= lds<COH>(s + 32 * (3 + 3 * e + v));
     }
   }
-  double* out = M.val + (row_start_ijk(P, c, i, j, k) + (int)hm[0] + (int)hm[1] + (int)hm[2]) * NB * NB;
+  BlockAt<NB> at;
+  if (live) at.set(M.val, row_start_ijk(P, c, i, j, k) + (int)hm[0] + (int)hm[1] + (int)hm[2]);
   bool ok = true;
 #pragma unroll
   for (int e = 0; e < NB; ++e) ok = ok && (!live || finite(r[e]));
   if (!ok) atomicOr(M.status, kStatNonFinite);
-  store_blocks<NB>(st, dg, live ? out : nullptr);
+  store_blocks<NB>(st, dg, M.val, at);
   if constexpr (NB == 3) {               // the warp's residuals are contiguous: stored in order
     const int lane = threadIdx.x & 31;
     const long long first = (c - lane) * NB, end = P.N * NB;

@@ -263,7 +263,9 @@ __global__ void __launch_bounds__(32) pn_reduce_kernel(Params P, const double* _
       }
     }
     if constexpr (NB == 3) __syncwarp();   // every lane has its block before the stage is written again
-    if (__any_sync(0xffffffffu, has[t])) store_blocks<NB>(st, out, base);
+    BlockAt<NB> at;
+    if (has[t]) at.set(val, slot);
+    if (__any_sync(0xffffffffu, has[t])) store_blocks<NB>(st, out, val, at);
   }
   if (live) {
     rr[0] = fma(-el[NB], scale, rr[0]);
