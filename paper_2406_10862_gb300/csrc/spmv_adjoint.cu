@@ -220,8 +220,9 @@ __global__ void __launch_bounds__(kSpmvThreads) spmv_grid_t_kernel(Params P, con
 // A 2x2 row is at most 7 x 32 bytes: 128-row tiles take 28.7 KB and leave
 // the SM at full occupancy.  With 3x3 blocks (504 bytes a row) shared memory
 // would cap residency near 14 warps per SM, and the register kernel above is
-// faster there (measured 28.6 against 30.5 us at 200 000 rows, while 2x2 at
-// 1.12 M rows took 60 against 74 us).  Same FMAs in the same order as
+// faster there (measured 28.6 against 30.5 us at 200 000 rows, later 25.3
+// against 27.8 with one-warp CTAs on both sides, while 2x2 at 1.12 M rows took
+// 60 against 74 us).  Same FMAs in the same order as
 // spmv_grid_kernel, so the two give identical bits.
 //
 // Bounds: the CTA's blocks occupy bytes [b0 B, b1 B) of val (B = 8 NB^2).
