@@ -54,17 +54,17 @@ def env_int(name, default):
 #   dram_bytes          DRAM read + write bytes of one call on the
 #                       100x100x20 workload
 STORED = {
-    "spmv": {"sources": ["spmv_adjoint.cu", "ocp_internal.cuh"], "sha16": "f3457da1c16ec428",
-             "dram_bytes": 104.44e6, "fp64_inst_per_cell": 63.84, "fp64_warp_inst_per_cell": 2.0041},
+    "spmv": {"sources": ["spmv_adjoint.cu", "block_io.cuh", "ocp_internal.cuh"], "sha16": "0dfe122329b53732",
+             "dram_bytes": 104.39e6, "fp64_inst_per_cell": 63.84, "fp64_warp_inst_per_cell": 2.0041},
     # FP64 counts: the three stage kernels' sum (the one-launch ordered kernel
-    # executes 372.54 / 12.0007).  DRAM bytes per call by launch mode
-    # ("ordered" of the launch shape): 0 with 128/128/256-cell tiles, 1 and 2
+    # executes 287.88 / 9.1505).  DRAM bytes per call by launch mode
+    # ("ordered" of the launch shape): 0 with 64/32/32-cell tiles, 1 and 2
     # with 64-cell tiles
-    "linearize": {"sources": ["linearize.cu", "ocp_internal.cuh"], "sha16": "630f544f6f1a0b3a",
-                  "fp64_inst_per_cell": 370.54, "fp64_warp_inst_per_cell": 11.9382,
-                  "dram_bytes": {"0": 326.81e6, "1": 204.19e6, "2": 121.56e6}},
-    "vjp": {"sources": ["spmv_adjoint.cu", "ocp_internal.cuh"], "sha16": "f3457da1c16ec428",
-            "fp64_inst_per_cell": 177.19, "fp64_warp_inst_per_cell": 5.5739, "dram_bytes": 147.39e6},
+    "linearize": {"sources": ["linearize.cu", "block_io.cuh", "ocp_internal.cuh"], "sha16": "914ef6a61c09e92f",
+                  "fp64_inst_per_cell": 285.88, "fp64_warp_inst_per_cell": 9.0880,
+                  "dram_bytes": {"0": 296.44e6, "1": 178.15e6, "2": 132.09e6}},
+    "vjp": {"sources": ["spmv_adjoint.cu", "block_io.cuh", "ocp_internal.cuh"], "sha16": "0dfe122329b53732",
+            "fp64_inst_per_cell": 172.19, "fp64_warp_inst_per_cell": 5.4177, "dram_bytes": 148.14e6},
 }
 
 
@@ -673,7 +673,7 @@ def lin_line(N, nnzb, ms, shape, shape_src, hbm_peak):
                     "traffic": traffic, "traffic_over_algorithmic": traffic / alg if traffic else None,
                     "traffic_by_launch_mode": {m: {"bytes": b, "over_algorithmic": b / alg}
                                                for m, b in sorted(by_mode.items())} or None,
-                    "traffic_launch_modes": "0: three launches, 128/128/256-cell tiles; 1: cell launch + ordered "
+                    "traffic_launch_modes": "0: three launches, 64/32/32-cell tiles; 1: cell launch + ordered "
                                             "face/assembly launch, 64-cell tiles; 2: one ordered launch, 64-cell "
                                             "tiles"},
             "fp64": fp64_part(stored("linearize", "fp64_inst_per_cell"),
