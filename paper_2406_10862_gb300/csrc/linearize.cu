@@ -108,8 +108,9 @@ __device__ __forceinline__ void discard_scratch(double* s, long long N, long lon
 }
 
 // One cell with its state loaded; SAT: its oil is saturated (as every cell's
-// of the warp).  The quantities go to scratch as soon as they are complete and
-// the rare well terms read them back, so that few values are held at a time.
+// of the warp).  The quantities go to scratch as soon as they are complete,
+// and the rare well terms wait there for the own terms they are subtracted
+// from, so that few values are held at a time.
 template <int NB, bool SAT>
 __device__ __forceinline__ void cell_terms(const ModelArgs& M, const Table& T, double* s, double pn, double swn,
                                            double xn, int fn, double po, double swo, double xo, int fo, double phs,
@@ -125,6 +126,20 @@ __device__ __forceinline__ void cell_terms(const ModelArgs& M, const Table& T, d
     cap_pressure<NB>(P, pn, k, q);
     dens_mob<NB, true, true, SAT>(P, f, k, q);
     store_q<NB>(s, q);
+    if (ip >= 0) {
+      double src[3], ds[3][3];
+      Perf w = M.perf[ip];
+      if (M.p_bh) w.p_bh = M.p_bh[w.well];
+      CellAux a{};
+      if (w.kind == 1) total_mob<NB>(P, f, k, true, a);
+      well_source<NB>(w, q, a, src, ds);
+#pragma unroll
+      for (int e = 0; e < NB; ++e) {
+        s[32 * (kSelf + e)] = src[e];
+#pragma unroll
+        for (int v = 0; v < NB; ++v) s[32 * (kSelf + 3 + 3 * e + v)] = ds[e][v];
+      }
+    }
   }
   double r[3], dg[3][3];
   if (!M.no_acc) {
@@ -146,22 +161,11 @@ __device__ __forceinline__ void cell_terms(const ModelArgs& M, const Table& T, d
     for (int e = 0; e < NB; ++e) r[e] = dg[e][0] = dg[e][1] = dg[e][2] = 0.0;
   }
   if (ip >= 0) {
-    double src[3], ds[3][3];
-    Perf w = M.perf[ip];
-    if (M.p_bh) w.p_bh = M.p_bh[w.well];
-    CellQ q;
-    load_q<NB>(s, q);
-    q.p = pn;
-    CellAux a{};
-    if (w.kind == 1) {
-      Kr k;
-      rel_perm<NB>(P, swn, f.sg, flag, k);
-      total_mob<NB>(P, f, k, true, a);
-    }
-    well_source<NB>(w, q, a, src, ds);
+#pragma unroll
     for (int e = 0; e < NB; ++e) {
-      r[e] = __dsub_rn(r[e], src[e]);
-      for (int v = 0; v < NB; ++v) dg[e][v] = __dsub_rn(dg[e][v], ds[e][v]);
+      r[e] = __dsub_rn(r[e], s[32 * (kSelf + e)]);
+#pragma unroll
+      for (int v = 0; v < NB; ++v) dg[e][v] = __dsub_rn(dg[e][v], s[32 * (kSelf + 3 + 3 * e + v)]);
     }
   }
 #pragma unroll
