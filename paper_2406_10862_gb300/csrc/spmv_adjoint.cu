@@ -338,13 +338,15 @@ __global__ void __launch_bounds__(kBulkRows) spmv_bulk_kernel(Params P, long lon
 }
 
 // ------------------------------------------------------------------ adjoint
-// One-warp CTAs with the PVT table read through L1: with a copy of the table in
-// shared memory they cost a copy per warp, and larger CTAs a coarser last wave
-// (100 000 cells: 39 us, against 40 and 43 with 64 and 128 threads and 44 with
-// 128 threads and the copy).
+// One-warp CTAs: larger ones leave a coarser last wave (100 000 cells: 39 us,
+// against 40 and 43 with 64 and 128 threads).  The PVT table is read through
+// L1; grids of fewer than two CTAs per SM, which wait for each of its
+// searches' probes, copy it to shared memory first (STAGED).  Through L1 /
+// staged: 300 cells 14.8 / 13.8 us, 8000 14.5 / 14.1 (two phases 9.2 / 9.0),
+// 20 000 14.9 / 14.8 (two phases 9.5 / 9.8), 50 000 22.3 / 25.6 (12.7 / 14.0).
 constexpr int kVjpThreads = 32;
 
-template <int NB>
+template <int NB, bool STAGED>
 __global__ void __launch_bounds__(kVjpThreads) vjp_kernel(Params P, const Table* __restrict__ gT,
                                                   const double* __restrict__ u_new,
                                                   const int8_t* __restrict__ f_new,
@@ -358,9 +360,17 @@ __global__ void __launch_bounds__(kVjpThreads) vjp_kernel(Params P, const Table*
                                                   const Perf* __restrict__ perf, double scale,
                                                   const double* __restrict__ lam,
                                                   double* __restrict__ g_unew, double* __restrict__ g_uold,
-                                                  double* __restrict__ g_lnk, double* __restrict__ g_phi) {
+                                                  double* __restrict__ g_lnk, double* __restrict__ g_phi,
+                                                  int* __restrict__ status) {
   pdl_wait();
-  const Table& T = *gT;
+  __shared__ __align__(16) unsigned char buf[STAGED ? sizeof(Table) : 16];
+  Table& sT = *reinterpret_cast<Table*>(buf);
+  if constexpr (STAGED) {
+    __shared__ unsigned long long bar;
+    unsigned uses = 0;
+    load_table(sT, gT, bar, uses, status);
+  }
+  const Table& T = STAGED ? sT : *gT;
   const long long N = P.N;
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c >= N) return;
@@ -507,15 +517,13 @@ cudaError_t launch_vjp(const ocp_grid* g, const double* u_new, const int8_t* f_n
   const Params& P = g->prm;
   const unsigned blocks = (unsigned)((P.N + kVjpThreads - 1) / kVjpThreads);
   const double scale = P.vol_rb / dt;
-  if (P.nb == 3)
-    return launch_pdl(vjp_kernel<3>, blocks, kVjpThreads, 0, s, P, (const Table*)g->d_table, u_new, f_new, u_old,
-                      f_old, (const double*)g->d_phi, val, face_flux, (const double*)g->d_wlnk,
-                      (const int32_t*)g->d_perf_of_cell, (const Perf*)g->d_perf, scale, lam, g_unew, g_uold, g_lnk,
-                      g_phi);
-  return launch_pdl(vjp_kernel<2>, blocks, kVjpThreads, 0, s, P, (const Table*)g->d_table, u_new, f_new, u_old,
-                    f_old, (const double*)g->d_phi, val, face_flux, (const double*)g->d_wlnk,
+  const bool staged = P.N < 2LL * kVjpThreads * g->sms;
+  const auto kernel = P.nb == 3 ? (staged ? vjp_kernel<3, true> : vjp_kernel<3, false>)
+                                : (staged ? vjp_kernel<2, true> : vjp_kernel<2, false>);
+  return launch_pdl(kernel, blocks, kVjpThreads, 0, s, P, (const Table*)g->d_table, u_new, f_new, u_old, f_old,
+                    (const double*)g->d_phi, val, face_flux, (const double*)g->d_wlnk,
                     (const int32_t*)g->d_perf_of_cell, (const Perf*)g->d_perf, scale, lam, g_unew, g_uold, g_lnk,
-                    g_phi);
+                    g_phi, g->d_status);
 }
 
 cudaError_t launch_well_rates(const ocp_grid* g, const double* u, const int8_t* flag, double* q,
