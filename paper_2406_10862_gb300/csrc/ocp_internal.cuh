@@ -96,14 +96,15 @@ inline int tile_index(int tpb) {
 }
 // Default launch shape of one grid of N cells on an SM count `sms`.  One warp
 // per CTA for the face and assembly stages: their warps share nothing, and
-// the finer CTAs leave a smaller last wave (200 000 cells: 163 us, against
-// 168 with 64-cell and 173 with 128/128/256-cell tiles; 50 000: 46 against 49
-// and 50; 1 M: 750 against 755 and 763).  The cell stage's CTAs copy the PVT
+// the finer CTAs leave a smaller last wave (200 000 cells: 149 us, against
+// 151 with 64-cell and 154 with 128/128/256-cell tiles; 50 000: 42 against 44
+// and 45; 1 M: 687 against 684 and 689).  The cell stage's CTAs copy the PVT
 // table, so they hold 64 cells where that still gives every SM two of them.
 // Grids of fewer than four 32-cell tiles per SM take the face stage split by
 // direction and the assembly by equation, since their time is their warps'
-// FP64 instruction count, not the SMs' throughput (10 000 cells: 23 against 28
-// us; 20 000: 29 against 29; 30 000: 42 against 34), and a grid of at most
+// FP64 instruction count, not the SMs' throughput (8000 cells: 21 against 27
+// us; 18 000: 26.4 against 27.6; 20 000: 28.2 against 27.8; 30 000: 41 against
+// 31; two phases 12 000: 14.9 against 15.2), and a grid of at most
 // `max_cluster` 32-cell tiles runs all three stages in one cluster launch.
 inline LaunchCfg default_cfg(long long N, int sms, int max_cluster = 0) {
   LaunchCfg c;
