@@ -1,10 +1,12 @@
 /*
- * ocp_probe.h -- measurement utility of the GB300 linearisation library.
+ * ocp_probe.h -- measurement and test aids of the GB300 linearisation library.
  *
- * The paper has no counterpart: this entry point measures the sustained FP64
+ * The paper has no counterpart.  ocp_probe_fp64 measures the sustained FP64
  * fused-multiply-add rate of a device, the denominator of the roofline of
  * the library's FP64-bound kernels (on GB300 the FP64 pipe, not HBM, bounds
- * the linearisation, the block-CSR product and the adjoint).
+ * the linearisation, the block-CSR product and the adjoint);
+ * ocp_probe_solver_limits lets a small grid run the solver's forms that only
+ * large grids, small devices or failures reach.
  */
 #ifndef OCP_PROBE_H
 #define OCP_PROBE_H
@@ -24,6 +26,15 @@ extern "C" {
  * Allocates and frees a small device buffer; synchronises the device.
  * Returns OCP_ERR_INVALID_ARG for a NULL output or reps < 1. */
 ocp_status ocp_probe_fp64(int device, int reps, double* dfma_per_s);
+
+/* Limits of the ocp_bicgstab* calls on one grid. */
+typedef struct ocp_solver_limits {
+  int polls;       /* polls of one wait between CTAs; 0: the library's own */
+  int short_cta;   /* the CTA of a cooperative launch whose waits all give up at once; -1: none */
+} ocp_solver_limits;
+
+/* Sets the limits of later solves on the grid; NULL restores the library's own. */
+ocp_status ocp_probe_solver_limits(ocp_grid* grid, const ocp_solver_limits* limits);
 
 #ifdef __cplusplus
 }

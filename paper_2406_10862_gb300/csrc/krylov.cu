@@ -29,7 +29,8 @@
 // (With one set of slots that all CTAs polled, 152 CTAs kept its few lines so
 // busy that a barrier took 4.8 us, against 1.4 us among 8 CTAs; with inboxes
 // 2.5 us.)  The launch is cooperative (all CTAs are resident); the waits are
-// bounded.  Small systems run as one thread-block cluster instead, with the
+// bounded, and a CTA whose wait runs out leaves without its part of x, so a
+// solve counts as finished only when every CTA has stored its part.  Small systems run as one thread-block cluster instead, with the
 // hardware's barrier and sums through distributed shared memory.
 #include <cmath>
 
@@ -56,9 +57,10 @@ constexpr int kClusterSmem = 120 * 1024;   // above half an SM's: the cluster's 
 // slots per CTA, [CTA][barrier parity][value][sender].  The barriers' numbers
 // go on from one solve to the next, so nothing is cleared in between.
 struct SolveResult {
-  double finished, iterations, rr, bb;
+  double iterations, rr, bb;
   unsigned long long epoch;
-  double pad[3];
+  unsigned stored;                     // CTAs that ended the loop and stored their x
+  unsigned pad[7];
 };
 struct alignas(16) Slot {
   double v;
@@ -83,6 +85,8 @@ struct SolveArgs {
   SolveResult* result;
   Slot* inbox;
   unsigned long long epoch;            // number of the last barrier of earlier solves
+  unsigned polls;                      // of one wait, after which it gives up
+  int short_cta;                       // CTA whose waits all give up at once (a test's), or -1
   int* status;
 };
 
@@ -490,8 +494,13 @@ __device__ __forceinline__ bool grid_wait(const SolveArgs& A, Shared& sh, unsign
   if (tid < nv * G) {
     const Slot* in = inbox_of(A, epoch, blockIdx.x, 0);    // the values' slots are consecutive
     double v[kPer];
+    const unsigned polls = (int)blockIdx.x == A.short_cta ? 0u : A.polls;
     unsigned it = 0;
-    for (bool all = false; !all;) {
+    for (bool all = false; !all; ++it) {
+      if (it == polls) {
+        ok = false;
+        break;
+      }
       all = slot_load(in + tid, v[0]) == epoch;
       if (nv * G > T) {                  // the others' loads in flight together
         unsigned long long got[kPer];
@@ -499,10 +508,6 @@ __device__ __forceinline__ bool grid_wait(const SolveArgs& A, Shared& sh, unsign
         for (int j = 1; j < kPer; ++j) got[j] = tid + j * T < nv * G ? slot_load(in + tid + j * T, v[j]) : epoch;
 #pragma unroll
         for (int j = 1; j < kPer; ++j) all = all && got[j] == epoch;
-      }
-      if (!all && ++it == kSpin) {
-        ok = false;
-        break;
       }
     }
     if constexpr (NV > 0) {
@@ -694,8 +699,8 @@ __global__ void __launch_bounds__(kSolveThreads, 1) solve_kernel(const __grid_co
     A.result->rr = rr;
     A.result->bb = bb;
     A.result->epoch = epoch;
-    A.result->finished = 1.0;
   }
+  if (tid == 0) atomicAdd(&A.result->stored, 1u);
 }
 
 template <int NB, bool WELLS>
@@ -780,6 +785,8 @@ ocp_status bicgstab_run(ocp_grid* g, const double* val, const WellSchur* ws, con
   A.result = (SolveResult*)g->d_solve_sync;
   A.inbox = (Slot*)(A.result + 1);
   A.epoch = g->solve_epoch;
+  A.polls = g->solve_test.polls > 0 ? (unsigned)g->solve_test.polls : kSpin;
+  A.short_cta = g->solve_test.short_cta;
   A.status = g->d_status;
   const WellSchur wsv = ws ? *ws : WellSchur{nullptr, nullptr, nullptr};
   if (e == cudaSuccess) e = cudaMemsetAsync(g->d_solve_sync, 0, sizeof(SolveResult), s);
@@ -818,9 +825,10 @@ ocp_status bicgstab_run(ocp_grid* g, const double* val, const WellSchur* ws, con
   SolveResult h{};
   if (e == cudaSuccess) e = cudaMemcpyAsync(&h, g->d_solve_sync, sizeof(h), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  g->solve_epoch = e == cudaSuccess && h.finished != 0.0 ? h.epoch : 0;
+  const bool finished = h.stored == (unsigned)A.ctas;
+  g->solve_epoch = e == cudaSuccess && finished ? h.epoch : 0;
   if (e != cudaSuccess) return report(OCP_ERR_CUDA, "ocp_bicgstab: %s", cudaGetErrorString(e));
-  if (h.finished == 0.0) return report(OCP_ERR_TIMEOUT, "ocp_bicgstab: a bounded device wait expired");
+  if (!finished) return report(OCP_ERR_TIMEOUT, "ocp_bicgstab: a bounded device wait expired");
   const int it = (int)h.iterations;
   const double res = std::sqrt(h.rr), bnorm = std::sqrt(h.bb);
   const double target = rtol * (bnorm > 0.0 ? bnorm : 1.0);

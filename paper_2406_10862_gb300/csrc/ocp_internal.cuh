@@ -14,6 +14,7 @@
 #include <stdint.h>
 
 #include "../../include/ocp.h"
+#include "../../include/ocp_probe.h"
 
 namespace ocp {
 
@@ -146,6 +147,7 @@ struct ocp_grid {
   unsigned long long solve_epoch;   // number of the last barrier of the solves so far
   double* d_planes;          // its scaled off-diagonal blocks (null where they did not fit)
   int64_t planes_doubles;
+  ocp_solver_limits solve_test = {0, -1};   // ocp_probe_solver_limits
   int64_t scratch_doubles;
   ocp::LaunchCfg cfg;        // launch shape of the linearisation
   int sms;                   // SM count of the device

@@ -1,6 +1,8 @@
-// Sustained FP64 FMA rate of a device (see include/ocp_probe.h).
+// Sustained FP64 FMA rate of a device, and limits on a grid's solves (see
+// include/ocp_probe.h).
 #include "../../include/ocp_probe.h"
 #include "kernels.cuh"
+#include "ocp_internal.cuh"
 
 namespace {
 
@@ -65,5 +67,11 @@ extern "C" ocp_status ocp_probe_fp64(int device, int reps, double* dfma_per_s) {
   if (prev >= 0 && prev != device) cudaSetDevice(prev);
   if (e != cudaSuccess) return ocp::report(OCP_ERR_CUDA, "ocp_probe_fp64: %s", cudaGetErrorString(e));
   *dfma_per_s = best;
+  return OCP_OK;
+}
+
+extern "C" ocp_status ocp_probe_solver_limits(ocp_grid* g, const ocp_solver_limits* limits) {
+  if (!g) return ocp::report(OCP_ERR_INVALID_ARG, "grid is NULL");
+  g->solve_test = limits ? *limits : ocp_solver_limits{0, -1};
   return OCP_OK;
 }

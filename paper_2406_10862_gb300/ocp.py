@@ -26,7 +26,7 @@ STATUS_NAMES = {0: "OCP_OK", 1: "OCP_ERR_INVALID_ARG", 2: "OCP_ERR_CUDA", 3: "OC
 
 # Every symbol the header declares; the CPU tests check the library exports them.
 EXPORTS = ["ocp_grid_create", "ocp_grid_destroy", "ocp_grid_info", "ocp_bsr_pattern", "ocp_linearize",
-           "ocp_linearize_noalloc", "ocp_probe_fp64", "ocp_batch_create", "ocp_batch_destroy",
+           "ocp_linearize_noalloc", "ocp_probe_fp64", "ocp_probe_solver_limits", "ocp_batch_create", "ocp_batch_destroy",
            "ocp_batch_set_io", "ocp_batch_linearize", "ocp_batch_graph_launch", "ocp_batch_tune",
            "ocp_batch_set_shape", "ocp_batch_get_shape", "ocp_batch_get_status", "ocp_grid_set_shape",
            "ocp_grid_get_shape", "ocp_grid_cluster_tiles",
@@ -94,6 +94,11 @@ class _Shape(ctypes.Structure):
     _fields_ = [("cells_per_tile", ctypes.c_int * 3), ("ctas_per_sm", ctypes.c_int * 3), ("ordered", ctypes.c_int)]
 
 
+class SolverLimits(ctypes.Structure):
+    """``ocp_solver_limits``: what ``Grid.probe_solver_limits`` sets."""
+    _fields_ = [(n, ctypes.c_int) for n in ("polls", "short_cta")]
+
+
 _lib = None
 
 
@@ -124,6 +129,7 @@ def load(build_if_missing: bool = False):
     lib.ocp_well_rates.argtypes = [vp, vp, vp, vp, vp]
     lib.ocp_get_status.argtypes = [vp, vp]
     lib.ocp_probe_fp64.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_double)]
+    lib.ocp_probe_solver_limits.argtypes = [vp, ctypes.POINTER(SolverLimits)]
     lib.ocp_batch_create.argtypes = [ctypes.POINTER(vp), ctypes.c_int, ctypes.POINTER(vp)]
     lib.ocp_batch_destroy.argtypes = [vp]
     lib.ocp_batch_set_io.argtypes = [vp, ctypes.POINTER(_BatchIO)]
@@ -383,6 +389,14 @@ class Grid:
         if check:
             _check(st)
         return st, it.value, rr.value
+
+    def probe_solver_limits(self, **limits):
+        """Test aid (``ocp_probe_solver_limits``): limits of later solves on
+        this grid; those not given are the library's own."""
+        lim = SolverLimits(short_cta=-1)
+        for k, v in limits.items():
+            setattr(lim, k, v)
+        _check(load().ocp_probe_solver_limits(self._h, ctypes.byref(lim)))
 
     def newton_update(self, u, flag, du, scale, ds_max, du_max, nswitch, stream=None):
         _check(load().ocp_newton_update(self._h, _ptr(u), _ptr(flag), _ptr(du), float(scale), float(ds_max),
