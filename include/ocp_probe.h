@@ -31,6 +31,7 @@ ocp_status ocp_probe_fp64(int device, int reps, double* dfma_per_s);
 typedef struct ocp_solver_limits {
   int polls;       /* polls of one wait between CTAs; 0: the library's own */
   int short_cta;   /* the CTA of a cooperative launch whose waits all give up at once; -1: none */
+  int ctas;        /* CTAs of a cooperative launch at most, and no one-cluster launch; 0: as the device allows */
 } ocp_solver_limits;
 
 /* Sets the limits of later solves on the grid; NULL restores the library's own. */

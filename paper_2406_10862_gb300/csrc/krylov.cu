@@ -32,6 +32,8 @@
 // bounded, and a CTA whose wait runs out leaves without its part of x, so a
 // solve counts as finished only when every CTA has stored its part.  Small systems run as one thread-block cluster instead, with the
 // hardware's barrier and sums through distributed shared memory.
+#include <cuda.h>
+
 #include <cmath>
 
 #include "kernels.cuh"
@@ -703,10 +705,72 @@ __global__ void __launch_bounds__(kSolveThreads, 1) solve_kernel(const __grid_co
   if (tid == 0) atomicAdd(&A.result->stored, 1u);
 }
 
+// SMs that work on stream s can use: those of its green context where it has
+// one, else the device's `sms` (which is the share under MPS).
+int stream_sms(cudaStream_t s, int sms) {
+  struct Driver {
+    decltype(&cuStreamGetCtx_v2) context = nullptr;
+    decltype(&cuGreenCtxGetDevResource) resource = nullptr;
+    Driver() {
+      void *c = nullptr, *r = nullptr;
+      cudaDriverEntryPointQueryResult qc, qr;
+      if (cudaGetDriverEntryPointByVersion("cuStreamGetCtx", &c, 12050, cudaEnableDefault, &qc) == cudaSuccess &&
+          cudaGetDriverEntryPointByVersion("cuGreenCtxGetDevResource", &r, 12040, cudaEnableDefault, &qr) == cudaSuccess &&
+          qc == cudaDriverEntryPointSuccess && qr == cudaDriverEntryPointSuccess) {
+        context = (decltype(context))c;
+        resource = (decltype(resource))r;
+      } else {
+        cudaGetLastError();
+      }
+    }
+  };
+  static const Driver driver;            // no green contexts where the driver lacks the calls
+  CUcontext ctx;
+  CUgreenCtx green = nullptr;
+  CUdevResource res;
+  if (!driver.context || driver.context((CUstream)s, &ctx, &green) != CUDA_SUCCESS || !green ||
+      driver.resource(green, &res, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS)
+    return sms;
+  return (int)res.sm.smCount < sms ? (int)res.sm.smCount : sms;
+}
+
 template <int NB, bool WELLS>
 const void* solve_function(bool planes, bool cluster) {
   if (cluster) return (const void*)solve_kernel<NB, WELLS, true, true>;
   return planes ? (const void*)solve_kernel<NB, WELLS, true, false> : (const void*)solve_kernel<NB, WELLS, false, false>;
+}
+
+const void* solve_function_of(int nb, bool wells, bool planes, bool cluster) {
+  if (nb == 3) return wells ? solve_function<3, true>(planes, cluster) : solve_function<3, false>(planes, cluster);
+  if (nb == 2) return wells ? solve_function<2, true>(planes, cluster) : solve_function<2, false>(planes, cluster);
+  return solve_function<1, false>(planes, cluster);    // scalar systems have no well unknowns
+}
+
+// The kernel's attributes, set once for the grid, and the largest cluster of
+// it that the device runs (0: none).
+cudaError_t solve_cluster_limit(ocp_grid* g, int nb, bool wells, int* limit) {
+  int& known = g->solve_cluster[nb == 1 ? 0 : 1 + wells];
+  if (known < 0) {
+    const void* fn = solve_function_of(nb, wells, true, true);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemVecBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    for (int planes = 0; planes < 2 && e == cudaSuccess; ++planes)
+      e = cudaFuncSetAttribute(solve_function_of(nb, wells, planes != 0, false),
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemVecBytes);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kMaxClusterTiles);
+    cfg.blockDim = dim3(kSolveThreads);
+    cfg.dynamicSmemBytes = kClusterSmem;
+    int n = 0;
+    if (cudaOccupancyMaxPotentialClusterSize(&n, fn, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    known = n < kMaxClusterTiles ? n : kMaxClusterTiles;
+  }
+  *limit = known;
+  return cudaSuccess;
 }
 
 }  // namespace
@@ -759,14 +823,18 @@ ocp_status bicgstab_run(ocp_grid* g, const double* val, const WellSchur* ws, con
   SolveArgs A{};
   A.P = g->prm;
   A.n = (int)n;
-  const int most = g->max_cluster < kMaxClusterTiles ? g->max_cluster : kMaxClusterTiles;
-  const bool cluster = planes && most > 0 && n <= (long long)most * kClusterRange;
-  long long ctas = (n + kMinRange - 1) / kMinRange;
-  if (ctas > (cluster ? most : sms)) ctas = cluster ? most : sms;
-  A.range = (int)(((n + ctas - 1) / ctas + 31) / 32 * 32);
-  A.ctas = (int)((n + A.range - 1) / A.range);
-  const int threads = A.range < 128 ? 128 : (A.range < kSolveThreads ? A.range : kSolveThreads);
-  A.smem_vecs = kSmemVecBytes / (8 * A.range) < kVecs ? kSmemVecBytes / (8 * A.range) : kVecs;
+  int smem = 0, threads = 0;
+  // at most `most` CTAs, each with a range of whole warps
+  auto shape = [&](long long most) {
+    long long ctas = (n + kMinRange - 1) / kMinRange;
+    if (ctas > most) ctas = most;
+    A.range = (int)(((n + ctas - 1) / ctas + 31) / 32 * 32);
+    A.ctas = (int)((n + A.range - 1) / A.range);
+    threads = A.range < 128 ? 128 : (A.range < kSolveThreads ? A.range : kSolveThreads);
+    const long long fit = kSmemVecBytes / (8LL * A.range);
+    A.smem_vecs = fit < kVecs ? (int)fit : kVecs;
+    smem = 8 * A.smem_vecs * A.range;
+  };
   A.planes = planes;
   A.val = val;
   A.dinv = work + 8 * n;
@@ -796,32 +864,46 @@ ocp_status bicgstab_run(ocp_grid* g, const double* val, const WellSchur* ws, con
   if (e == cudaSuccess)
     e = launch_pdl(scale, blocks, 256, 0, s, g->prm, (int)n, val, A.trans, (const int32_t*)g->d_perf_of_cell,
                    (const Perf*)g->d_perf, wsv, b, planes, dinv, A.vec[0], wb, g->d_status);
-  const bool pl = planes != nullptr;
-  const void* fn = nb == 3   ? (ws ? solve_function<3, true>(pl, cluster) : solve_function<3, false>(pl, cluster))
-                   : nb == 2 ? (ws ? solve_function<2, true>(pl, cluster) : solve_function<2, false>(pl, cluster))
-                             : solve_function<1, false>(pl, cluster);     // scalar systems have no well unknowns
-  int smem = 8 * A.smem_vecs * A.range;
-  if (cluster && smem < kClusterSmem) smem = kClusterSmem;
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemVecBytes);
-  if (e == cudaSuccess && cluster) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   void* args[] = {&A};
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)A.ctas);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cfg.stream = s;
   cudaLaunchAttribute attr[1];
-  if (cluster) {
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)A.ctas;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-  } else {
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-  }
+  cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (e == cudaSuccess) e = cudaLaunchKernelExC(&cfg, fn, args);
+  auto launch = [&](bool cluster) {
+    if (cluster && smem < kClusterSmem) smem = kClusterSmem;
+    cfg.gridDim = dim3((unsigned)A.ctas);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    if (cluster) {
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = (unsigned)A.ctas;
+      attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    } else {
+      attr[0].id = cudaLaunchAttributeCooperative;
+      attr[0].val.cooperative = 1;
+    }
+    return cudaLaunchKernelExC(&cfg, solve_function_of(nb, ws != nullptr, planes != nullptr, cluster), args);
+  };
+  // One cluster where it takes the system and the stream has the whole device;
+  // else a cooperative launch of a CTA per SM that the stream can use, or of
+  // fewer where so many are refused.
+  const int use = stream_sms(s, sms), asked = g->solve_test.ctas;
+  int most = 0;
+  if (e == cudaSuccess) e = solve_cluster_limit(g, nb, ws != nullptr, &most);
+  bool launched = false;
+  if (e == cudaSuccess && planes && use == sms && asked == 0 && n <= (long long)most * kClusterRange) {
+    shape(most);
+    launched = launch(true) == cudaSuccess;
+    if (!launched) cudaGetLastError();
+  }
+  for (int ctas = asked > 0 && asked < use ? asked : use; e == cudaSuccess && !launched; ctas = A.ctas / 2) {
+    shape(ctas);
+    const cudaError_t el = launch(false);
+    launched = el == cudaSuccess;
+    if (el == cudaErrorCooperativeLaunchTooLarge && A.ctas > 1) cudaGetLastError();
+    else e = el;
+  }
   SolveResult h{};
   if (e == cudaSuccess) e = cudaMemcpyAsync(&h, g->d_solve_sync, sizeof(h), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);

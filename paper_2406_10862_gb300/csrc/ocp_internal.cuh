@@ -147,7 +147,8 @@ struct ocp_grid {
   unsigned long long solve_epoch;   // number of the last barrier of the solves so far
   double* d_planes;          // its scaled off-diagonal blocks (null where they did not fit)
   int64_t planes_doubles;
-  ocp_solver_limits solve_test = {0, -1};   // ocp_probe_solver_limits
+  int solve_cluster[3] = {-1, -1, -1};   // largest cluster of the scalar, block and well solver (-1: not asked yet)
+  ocp_solver_limits solve_test = {0, -1, 0};   // ocp_probe_solver_limits
   int64_t scratch_doubles;
   ocp::LaunchCfg cfg;        // launch shape of the linearisation
   int sms;                   // SM count of the device
