@@ -38,9 +38,9 @@
  *   sticky in the grid's status word and reported by ocp_get_status().
  * There is no CPU fallback: every compute call runs CUDA kernels for sm_103a.
  * Only ocp_grid_create, ocp_batch_create, their destroy calls, the first
- *   ocp_linearize_pn on a grid (its phase-split data) and the first
- *   ocp_bicgstab* of each block size (the solver's copy of the scaled matrix)
- *   allocate or free device memory.
+ *   ocp_linearize_pn on a grid (its phase-split data), ocp_solver_release and
+ *   an ocp_bicgstab* call that is lent no memory (the solver's copy of the
+ *   scaled matrix) allocate or free device memory.
  * ocp_last_error() returns a thread-local message describing the last failure.
  */
 #ifndef OCP_H
@@ -302,16 +302,29 @@ int64_t ocp_solver_work_doubles(const ocp_grid* grid);
  * on entry and the solution on return; b and x are block-interleaved [nb*N]
  * device vectors; work is a device buffer of ocp_solver_work_doubles().
  * The iterations run in one cooperative launch with the convergence test on
- * the device; the stream is synchronised once, at the end.  The grid keeps the
- * solver's copy of D^-1 A (6 nb^2 doubles per cell, 6 for a scalar system),
- * allocated by the first call; where it does not fit, the same iteration runs
- * from bsr_val itself.  Calls on one grid must not overlap from several host
- * threads.  The paper solves with CPR-preconditioned FGMRES in PETSc/Hypre
+ * the device; the stream is synchronised once, at the end.  The iteration reads
+ * the solver's copy of D^-1 A (6 nb^2 doubles per cell, 6 for a scalar system) in
+ * memory lent to the call (ocp_solver_lend), else in memory that the first call
+ * allocates and the grid keeps until ocp_solver_release; where neither has room
+ * for it, the same iteration runs, slower, from bsr_val itself.  Calls on one
+ * grid must not overlap from several host threads.  The paper solves with CPR-preconditioned FGMRES in PETSc/Hypre
  * (Sec. 5.1); this plain Krylov solver serves the Newton, adjoint and test
  * drivers.  Returns OCP_ERR_TIMEOUT when maxit is reached, OCP_ERR_NONFINITE on breakdown;
  * *iters and *relres (may be NULL) report the final state. */
 ocp_status ocp_bicgstab(ocp_grid* grid, const double* bsr_val, const double* b, double* x, double rtol,
                         int maxit, int transpose, double* work, int* iters, double* relres, void* cuda_stream);
+
+/* Size in doubles of the memory to lend a solve with block size nb (the grid's,
+ * or 1) for its copy of the matrix; 0 where the copy takes at most 1 MiB and has
+ * its place in the grid. */
+int64_t ocp_solver_matrix_doubles(const ocp_grid* grid, int nb);
+/* Lends the next ocp_bicgstab* call on the grid device memory for its copy of
+ * the matrix: that call allocates none, and the memory is the caller's again
+ * when it returns, whatever it returns.  With less than
+ * ocp_solver_matrix_doubles (0 and NULL: none) the call runs from bsr_val. */
+ocp_status ocp_solver_lend(ocp_grid* grid, double* buf, int64_t doubles);
+/* Frees what the grid keeps for solves that are lent nothing. */
+ocp_status ocp_solver_release(ocp_grid* grid);
 
 /* Newton update u += scale * du (du block-interleaved, u and flag as for
  * ocp_linearize; scale = -1 applies the solution of J x = R), with every

@@ -264,8 +264,9 @@ ocp_status ocp_grid_create(const ocp_grid_desc* d, int device, ocp_grid** out) {
   OCP_ALLOC(g->d_scratch, sizeof(double) * g->scratch_doubles);
   OCP_ALLOC(g->d_sync, sizeof(unsigned) * (1 + 2 * ((N + 31) / 32)));
   OCP_ALLOC(d_lnk, sizeof(double) * N);
-#undef OCP_ALLOC
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, device);
+  OCP_ALLOC(g->d_solve_sync, ocp::solver_own_bytes(g));
+#undef OCP_ALLOC
   // default launch shape (ocp_grid_set_shape and the batch autotuner can
   // change it): one CTA per tile, tiles as large as the grid's size allows
   g->cfg = ocp::default_cfg(N, g->sms);

@@ -348,6 +348,7 @@ ocp_status ocp_impec_update(ocp_grid* g, const double* pn_old, const double* dp,
 ocp_status ocp_bicgstab_scalar(ocp_grid* g, const double* val, const double* b, double* x, double rtol, int maxit,
                                double* work, int* iters, double* relres, void* stream) {
   using namespace ocp;
+  const LoanEnd loan(g);
   if (!g || !val || !b || !x || !work) return report(OCP_ERR_INVALID_ARG, "grid, val, b, x and work are required");
   if (b == x) return report(OCP_ERR_INVALID_ARG, "b and x must not overlap");
   Guard guard(g->device);

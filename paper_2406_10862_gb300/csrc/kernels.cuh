@@ -45,6 +45,17 @@ cudaError_t launch_well_back(const ocp_grid* g, const WellSchur& ws, const doubl
 ocp_status bicgstab_run(ocp_grid* g, const double* val, const WellSchur* ws, const double* b, double* x,
                         double rtol, int maxit, int transpose, double* work, int* iters, double* relres,
                         cudaStream_t s, int nbs = 0);
+size_t solver_own_bytes(const ocp_grid* g);
+// Held by every ocp_bicgstab* call: what was lent to it goes back, however it ends.
+struct LoanEnd {
+  ocp_grid* g;
+  explicit LoanEnd(ocp_grid* grid) : g(grid) {}
+  ~LoanEnd() {
+    if (!g) return;
+    g->lent = nullptr;
+    g->lent_doubles = -1;
+  }
+};
 void free_solver(ocp_grid* g);
 cudaError_t launch_tiles(int nb, const TileList* lists, const ModelArgs& single, const LaunchCfg& cfg,
                          int sms, cudaStream_t s);

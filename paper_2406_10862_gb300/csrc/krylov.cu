@@ -48,6 +48,10 @@ constexpr int kMaxCtas = 256;
 constexpr int kVecs = 7;               // r, r0, p, v, s, t, x
 constexpr unsigned kSpin = 1u << 21;   // polls of one slot, above a second
 constexpr int kSmemVecBytes = 213 * 1024;
+// A copy of the scaled matrix of at most so many doubles (1 MiB: 2427 cells
+// with 3x3 blocks) has its place beside the slots from the grid's creation on:
+// asking for memory in each solve cost a step of 300 cells 3 % of its time.
+constexpr int64_t kOwnPlanes = 1 << 17;
 // The one-cluster launch takes systems of at most so many unknowns per CTA of
 // the largest cluster.  Per iteration, cluster / cooperative launch: 300 cells
 // (3x3) 12.2 / 15.6 us, 1260 13.5 / 14.9, 1728 15.1 / 15.7, 2400 16.8 / 16.7;
@@ -302,9 +306,11 @@ __device__ __forceinline__ double row_z(const SolveArgs& A, const RowAt& w, int 
   return acc;
 }
 
-// The whole of it from the matrix itself and the block inverses, where the
-// planes could not be allocated: every thread forms the NB entries of its cell's
-// A x and applies its row of D^-1.
+// The whole of it from the matrix itself and the block inverses, where there is
+// no room for the planes: every thread forms the NB entries of its cell's A x
+// and applies its row of D^-1.  Per iteration, with the planes / without:
+// 100 000 cells (3x3) 44 / 82 us, 200 000 73 / 208, 400 000 131 / 402, 1 122 000
+// (2x2) 233 / 413.
 template <int NB>
 __device__ __noinline__ double row_product_unscaled(const SolveArgs& A, int i, const double* x) {
   constexpr int B2 = NB * NB;
@@ -775,6 +781,22 @@ cudaError_t solve_cluster_limit(ocp_grid* g, int nb, bool wells, int* limit) {
 
 }  // namespace
 
+int64_t planes_need(const ocp_grid* g, int nb) { return 6LL * nb * nb * g->prm.N; }
+
+// Results and slots of a solve with a CTA per SM, or per kMinRange unknowns
+// where that is fewer; then the place of a small copy of the matrix.
+size_t solver_sync_bytes(const ocp_grid* g) {
+  const long long need = (g->prm.nb * g->prm.N + kMinRange - 1) / kMinRange;
+  long long ctas = g->sms < kMaxCtas ? g->sms : kMaxCtas;
+  if (ctas > need) ctas = need;
+  return sizeof(SolveResult) + sizeof(Slot) * 6 * (size_t)(ctas * ctas);
+}
+size_t solver_own_bytes(const ocp_grid* g) {
+  const int64_t block = planes_need(g, g->prm.nb), scalar = planes_need(g, 1);
+  const int64_t own = block <= kOwnPlanes ? block : (scalar <= kOwnPlanes ? scalar : 0);
+  return solver_sync_bytes(g) + sizeof(double) * own;
+}
+
 int64_t solver_work_doubles(const ocp_grid* g) {
   const int64_t n = (int64_t)g->prm.nb * g->prm.N;
   // r, r0, p, v, s, t; the scaled well columns; the block inverses (used
@@ -782,9 +804,15 @@ int64_t solver_work_doubles(const ocp_grid* g) {
   return 9 * n + (int64_t)g->prm.nb * g->prm.nb * g->prm.N + 633;
 }
 
+void free_planes(ocp_grid* g) {
+  cudaFree(g->d_planes);
+  g->d_planes = nullptr;
+  g->planes_doubles = 0;
+}
+
 void free_solver(ocp_grid* g) {
   cudaFree(g->d_solve_sync);
-  cudaFree(g->d_planes);
+  free_planes(g);
 }
 
 ocp_status bicgstab_run(ocp_grid* g, const double* val, const WellSchur* ws, const double* b, double* x,
@@ -795,31 +823,27 @@ ocp_status bicgstab_run(ocp_grid* g, const double* val, const WellSchur* ws, con
   const long long N = g->prm.N, n = nb * N;
   cudaError_t e = cudaSuccess;
   const int sms = g->sms < kMaxCtas ? g->sms : kMaxCtas;
-  const size_t sync_bytes = sizeof(SolveResult) + sizeof(Slot) * 6 * (size_t)sms * sms;
-  if (!g->d_solve_sync) {
-    e = cudaMalloc((void**)&g->d_solve_sync, sync_bytes);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      g->d_solve_sync = nullptr;
-      return report(OCP_ERR_OOM, "ocp_bicgstab: %s", cudaGetErrorString(e));
-    }
-    g->solve_epoch = 0;
-  }
+  const size_t sync_bytes = solver_sync_bytes(g);
   // the slots start from zero, and again after a solve that did not finish
   if (g->solve_epoch == 0) e = cudaMemsetAsync(g->d_solve_sync, 0, sync_bytes, s);
-  const int64_t want = 6LL * nb * n;
-  if (g->planes_doubles < want) {
-    cudaFree(g->d_planes);
-    g->d_planes = nullptr;
-    g->planes_doubles = 0;
-    if (cudaMalloc((void**)&g->d_planes, sizeof(double) * want) == cudaSuccess) {
-      g->planes_doubles = want;
-    } else {                              // no room: solve from the matrix itself
-      cudaGetLastError();
-      g->d_planes = nullptr;
+  const int64_t want = planes_need(g, nb);
+  double* planes = nullptr;
+  if (want <= kOwnPlanes) {
+    planes = (double*)((char*)g->d_solve_sync + sync_bytes);
+  } else if (g->lent_doubles >= 0) {      // memory of the caller's, or none
+    if (g->lent && g->lent_doubles >= want) planes = g->lent;
+  } else {
+    if (g->planes_doubles < want) {
+      free_planes(g);
+      if (cudaMalloc((void**)&g->d_planes, sizeof(double) * want) == cudaSuccess) {
+        g->planes_doubles = want;
+      } else {                            // no room: solve from the matrix itself
+        cudaGetLastError();
+        g->d_planes = nullptr;
+      }
     }
+    if (g->planes_doubles >= want) planes = g->d_planes;
   }
-  double* planes = g->planes_doubles >= want ? g->d_planes : nullptr;
   SolveArgs A{};
   A.P = g->prm;
   A.n = (int)n;
@@ -923,3 +947,34 @@ ocp_status bicgstab_run(ocp_grid* g, const double* val, const WellSchur* ws, con
 }
 
 }  // namespace ocp
+
+extern "C" {
+
+int64_t ocp_solver_matrix_doubles(const ocp_grid* g, int nb) {
+  if (!g || (nb != 1 && nb != g->prm.nb)) return 0;
+  const int64_t n = ocp::planes_need(g, nb);
+  return n <= ocp::kOwnPlanes ? 0 : n;
+}
+
+ocp_status ocp_solver_lend(ocp_grid* g, double* buf, int64_t doubles) {
+  using namespace ocp;
+  if (!g || doubles < 0 || (!buf && doubles > 0))
+    return report(OCP_ERR_INVALID_ARG, "grid, a buffer and its size are required");
+  g->lent = buf;
+  g->lent_doubles = doubles;
+  return OCP_OK;
+}
+
+ocp_status ocp_solver_release(ocp_grid* g) {
+  using namespace ocp;
+  if (!g) return report(OCP_ERR_INVALID_ARG, "grid is NULL");
+  int prev = -1;
+  cudaError_t e = cudaGetDevice(&prev);
+  if (e == cudaSuccess && prev != g->device) e = cudaSetDevice(g->device);
+  if (e != cudaSuccess) return report(OCP_ERR_CUDA, "cudaSetDevice: %s", cudaGetErrorString(e));
+  free_planes(g);
+  if (prev != g->device) cudaSetDevice(prev);
+  return OCP_OK;
+}
+
+}  // extern "C"

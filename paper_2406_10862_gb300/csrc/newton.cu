@@ -141,6 +141,7 @@ int64_t ocp_solver_work_doubles(const ocp_grid* g) { return g ? ocp::solver_work
 ocp_status ocp_bicgstab(ocp_grid* g, const double* val, const double* b, double* x, double rtol, int maxit,
                         int transpose, double* work, int* iters, double* relres, void* stream) {
   using namespace ocp;
+  const LoanEnd loan(g);
   if (!g || !val || !b || !x || !work) return report(OCP_ERR_INVALID_ARG, "grid, val, b, x and work are required");
   if (b == x) return report(OCP_ERR_INVALID_ARG, "b and x must not overlap");
   Guard guard(g->device);

@@ -143,10 +143,12 @@ struct ocp_grid {
   unsigned* d_sync;          // ordered launch: item counter, then cell and face flags per 32-cell tile
   double* d_pn;              // per-cell data of the (P, N) path, allocated on its first use
   int8_t* d_pn_flag;
-  void* d_solve_sync;        // the solver's results and barrier slots, allocated by the first solve
+  void* d_solve_sync;        // the solver's results and barrier slots, and its copy of a small matrix
   unsigned long long solve_epoch;   // number of the last barrier of the solves so far
-  double* d_planes;          // its scaled off-diagonal blocks (null where they did not fit)
-  int64_t planes_doubles;
+  double* d_planes;          // its scaled off-diagonal blocks (null where they did not fit), for solves
+  int64_t planes_doubles;    // that are lent no memory
+  double* lent;              // memory lent to the next solve; lent_doubles < 0: none was
+  int64_t lent_doubles = -1;
   int solve_cluster[3] = {-1, -1, -1};   // largest cluster of the scalar, block and well solver (-1: not asked yet)
   ocp_solver_limits solve_test = {0, -1, 0};   // ocp_probe_solver_limits
   int64_t scratch_doubles;

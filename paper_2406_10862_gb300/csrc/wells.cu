@@ -270,6 +270,7 @@ ocp_status ocp_bicgstab_wells(ocp_grid* g, const double* val, const double* well
                               double rtol, int maxit, int transpose, double* work, int* iters, double* relres,
                               void* stream) {
   using namespace ocp;
+  const LoanEnd loan(g);
   if (!g || !val || !b || !x || !work) return report(OCP_ERR_INVALID_ARG, "grid, val, b, x and work are required");
   if (g->nwell == 0) return ocp_bicgstab(g, val, b, x, rtol, maxit, transpose, work, iters, relres, stream);
   if (!well_d || !b_w || !x_w || (g->nperf > 0 && (!well_b || !well_c)))

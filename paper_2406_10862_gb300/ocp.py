@@ -11,8 +11,10 @@ The functions keep the C names (``ocp_linearize`` ...); ``Grid`` wraps them.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
+import warnings
 
 import numpy as np
 import torch
@@ -30,7 +32,8 @@ EXPORTS = ["ocp_grid_create", "ocp_grid_destroy", "ocp_grid_info", "ocp_bsr_patt
            "ocp_batch_set_io", "ocp_batch_linearize", "ocp_batch_graph_launch", "ocp_batch_tune",
            "ocp_batch_set_shape", "ocp_batch_get_shape", "ocp_batch_get_status", "ocp_grid_set_shape",
            "ocp_grid_get_shape", "ocp_grid_cluster_tiles",
-           "ocp_solver_work_doubles", "ocp_bicgstab", "ocp_newton_update", "ocp_well_rates_vjp",
+           "ocp_solver_work_doubles", "ocp_solver_matrix_doubles", "ocp_solver_lend", "ocp_solver_release",
+           "ocp_bicgstab", "ocp_newton_update", "ocp_well_rates_vjp",
            "ocp_grid_update_perm", "ocp_coupling_work_ints", "ocp_coupling_components", "ocp_linearize_wells",
            "ocp_bicgstab_wells", "ocp_well_update", "ocp_residual_norms", "ocp_linearize_pn", "ocp_pn_update",
            "ocp_pn_norms", "ocp_pn_from_natural", "ocp_impec_pressure", "ocp_impec_update", "ocp_bicgstab_scalar", "ocp_bsr_spmv", "ocp_adjoint_vjp",
@@ -144,6 +147,10 @@ def load(build_if_missing: bool = False):
     lib.ocp_grid_cluster_tiles.argtypes = [vp, ctypes.POINTER(ctypes.c_int)]
     lib.ocp_solver_work_doubles.argtypes = [vp]
     lib.ocp_solver_work_doubles.restype = ctypes.c_int64
+    lib.ocp_solver_matrix_doubles.argtypes = [vp, ctypes.c_int]
+    lib.ocp_solver_matrix_doubles.restype = ctypes.c_int64
+    lib.ocp_solver_lend.argtypes = [vp, vp, ctypes.c_int64]
+    lib.ocp_solver_release.argtypes = [vp]
     lib.ocp_bicgstab.argtypes = [vp, vp, vp, vp, ctypes.c_double, ctypes.c_int, ctypes.c_int, vp,
                                  ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_double), vp]
     lib.ocp_newton_update.argtypes = [vp, vp, vp, vp, ctypes.c_double, ctypes.c_double, vp, vp, vp]
@@ -169,7 +176,8 @@ def load(build_if_missing: bool = False):
                                             ctypes.c_int, vp, vp, vp]
     lib.ocp_last_error.restype = ctypes.c_char_p
     for name in EXPORTS:
-        if name not in ("ocp_last_error", "ocp_solver_work_doubles", "ocp_coupling_work_ints"):
+        if name not in ("ocp_last_error", "ocp_solver_work_doubles", "ocp_solver_matrix_doubles",
+                        "ocp_coupling_work_ints"):
             getattr(lib, name).restype = ctypes.c_int
     _lib = lib
     return lib
@@ -253,6 +261,8 @@ class Grid:
         with torch.cuda.device(self.device):
             _check(lib.ocp_grid_create(ctypes.byref(d), self.device.index or 0, ctypes.byref(h)))
         self._h = h
+        self._copy = {}                      # doubles to lend a solve, by block size
+        self._short = False                  # the last solve found no room for them
         del keep
         n, nb, nnzb = ctypes.c_int64(), ctypes.c_int(), ctypes.c_int64()
         _check(lib.ocp_grid_info(h, ctypes.byref(n), ctypes.byref(nb), ctypes.byref(nnzb)))
@@ -378,11 +388,39 @@ class Grid:
     def solver_work(self):
         return self.empty(int(load().ocp_solver_work_doubles(self._h)))
 
+    def _lend(self, nb, stream):
+        """Lends the next solve memory of torch's for its copy of a large matrix,
+        taken on the solve's stream and returned here (keep it until the solve,
+        which synchronises, is over); None, with a warning, where there is no
+        room: the solve then runs slower from the matrix itself.  After that
+        torch is asked again only once the memory is there, since an allocation
+        that fails empties its cache."""
+        n = self._copy.get(nb)
+        if n is None:
+            n = self._copy[nb] = int(load().ocp_solver_matrix_doubles(self._h, nb))
+        if n == 0:
+            return None
+        buf = None
+        if not self._short or self._free_bytes() >= 8 * n + (32 << 20):
+            try:
+                with torch.cuda.stream(stream) if stream is not None else contextlib.nullcontext():
+                    buf = self.empty(n)
+            except torch.OutOfMemoryError:
+                warnings.warn("no room for %d bytes: the solver runs from the matrix itself" % (8 * n), RuntimeWarning)
+            self._short = buf is None
+        _check(load().ocp_solver_lend(self._h, _ptr(buf), n if buf is not None else 0))
+        return buf
+
+    def _free_bytes(self):
+        return (torch.cuda.mem_get_info(self.device)[0] + torch.cuda.memory_reserved(self.device)
+                - torch.cuda.memory_allocated(self.device))
+
     def bicgstab(self, bsr_val, b, x, rtol, maxit, transpose=False, work=None, stream=None, check=True):
         """Solve A x = b (A^T x = b); x is the initial guess, updated in place.
         Returns (status, iterations, relative residual)."""
         work = work if work is not None else self.solver_work()
         it, rr = ctypes.c_int(), ctypes.c_double()
+        lent = self._lend(self.nb, stream)  # noqa: F841 -- held until the solve is over
         st = load().ocp_bicgstab(self._h, _ptr(bsr_val), _ptr(b), _ptr(x), float(rtol), int(maxit),
                                  int(bool(transpose)), _ptr(work), ctypes.byref(it), ctypes.byref(rr),
                                  _stream(self.device, stream))
@@ -446,6 +484,7 @@ class Grid:
         guess.  Returns (status, iterations, relative residual)."""
         work = work if work is not None else self.solver_work()
         it, rr = ctypes.c_int(), ctypes.c_double()
+        lent = self._lend(self.nb, stream)  # noqa: F841 -- held until the solve is over
         st = load().ocp_bicgstab_wells(self._h, _ptr(bsr_val), _ptr(well_b), _ptr(well_c), _ptr(well_d), _ptr(b),
                                        _ptr(b_w), _ptr(x), _ptr(x_w), float(rtol), int(maxit),
                                        int(bool(transpose)), _ptr(work), ctypes.byref(it), ctypes.byref(rr),
@@ -522,6 +561,7 @@ class Grid:
     def bicgstab_scalar(self, val, b, x, rtol, maxit, work=None, stream=None, check=True):
         work = work if work is not None else self.solver_work()
         it, rr = ctypes.c_int(), ctypes.c_double()
+        lent = self._lend(1, stream)  # noqa: F841 -- held until the solve is over
         st = load().ocp_bicgstab_scalar(self._h, _ptr(val), _ptr(b), _ptr(x), float(rtol), int(maxit), _ptr(work),
                                         ctypes.byref(it), ctypes.byref(rr), _stream(self.device, stream))
         if check:
