@@ -32,6 +32,7 @@ typedef struct ocp_solver_limits {
   int polls;       /* polls of one wait between CTAs; 0: the library's own */
   int short_cta;   /* the CTA of a cooperative launch whose waits all give up at once; -1: none */
   int ctas;        /* CTAs of a cooperative launch at most, and no one-cluster launch; 0: as the device allows */
+  int spill;       /* of the seven vectors that a CTA keeps in shared memory, how many stay in global memory instead */
 } ocp_solver_limits;
 
 /* Sets the limits of later solves on the grid; NULL restores the library's own. */

@@ -856,7 +856,8 @@ ocp_status bicgstab_run(ocp_grid* g, const double* val, const WellSchur* ws, con
     A.ctas = (int)((n + A.range - 1) / A.range);
     threads = A.range < 128 ? 128 : (A.range < kSolveThreads ? A.range : kSolveThreads);
     const long long fit = kSmemVecBytes / (8LL * A.range);
-    A.smem_vecs = fit < kVecs ? (int)fit : kVecs;
+    A.smem_vecs = (fit < kVecs ? (int)fit : kVecs) - g->solve_test.spill;
+    if (A.smem_vecs < 0) A.smem_vecs = 0;
     smem = 8 * A.smem_vecs * A.range;
   };
   A.planes = planes;

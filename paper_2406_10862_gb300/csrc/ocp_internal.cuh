@@ -150,7 +150,7 @@ struct ocp_grid {
   double* lent;              // memory lent to the next solve; lent_doubles < 0: none was
   int64_t lent_doubles = -1;
   int solve_cluster[3] = {-1, -1, -1};   // largest cluster of the scalar, block and well solver (-1: not asked yet)
-  ocp_solver_limits solve_test = {0, -1, 0};   // ocp_probe_solver_limits
+  ocp_solver_limits solve_test = {0, -1, 0, 0};   // ocp_probe_solver_limits
   int64_t scratch_doubles;
   ocp::LaunchCfg cfg;        // launch shape of the linearisation
   int sms;                   // SM count of the device

@@ -72,6 +72,6 @@ extern "C" ocp_status ocp_probe_fp64(int device, int reps, double* dfma_per_s) {
 
 extern "C" ocp_status ocp_probe_solver_limits(ocp_grid* g, const ocp_solver_limits* limits) {
   if (!g) return ocp::report(OCP_ERR_INVALID_ARG, "grid is NULL");
-  g->solve_test = limits ? *limits : ocp_solver_limits{0, -1, 0};
+  g->solve_test = limits ? *limits : ocp_solver_limits{0, -1, 0, 0};
   return OCP_OK;
 }

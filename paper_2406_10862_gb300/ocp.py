@@ -99,7 +99,7 @@ class _Shape(ctypes.Structure):
 
 class SolverLimits(ctypes.Structure):
     """``ocp_solver_limits``: what ``Grid.probe_solver_limits`` sets."""
-    _fields_ = [(n, ctypes.c_int) for n in ("polls", "short_cta", "ctas")]
+    _fields_ = [(n, ctypes.c_int) for n in ("polls", "short_cta", "ctas", "spill")]
 
 
 _lib = None
