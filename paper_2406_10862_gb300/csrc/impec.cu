@@ -14,8 +14,9 @@
 //   impec_update_kernel  per cell: the face fluxes and well terms at the new
 //                        pressure and N^{n+1} = N^n + (Q - sum F) dt / V.
 // A face's flux seen from its two cells is the exact negation of the same
-// floating-point expression, so the update conserves every component to
-// rounding.
+// floating-point expression -- at a potential difference of zero both take the
+// lower-numbered cell as upstream -- so the update conserves every component
+// to rounding.
 #include <cmath>
 
 #include "kernels.cuh"
@@ -100,22 +101,24 @@ __device__ __forceinline__ void impec_load(const double* d, bool z, ImpecSide<NB
   f.rs = NB == 3 ? d[32 * kRs] : 0.0;
 }
 
-// One face from the row cell (c) to its neighbour (n): per phase the frozen
-// coefficient T lambda_up and the old potential difference, and the oil's
-// upwind R_s.
+// One face from the row cell (c) to its neighbour (n; `minus`: the lower-numbered
+// one): per phase the frozen coefficient T lambda_up and the old potential
+// difference, and the oil's upwind R_s.  Upstream is the lower-numbered cell
+// where the potential does not grow from it, so the row of the other one is
+// upstream only where its own potential is strictly the higher.
 template <int NB>
 struct FaceCoef {
   double c[NB], dphi[NB], rs_up;
 };
 template <int NB>
-__device__ __forceinline__ void face_coef(const ImpecSide<NB>& c, const ImpecSide<NB>& n, bool z, double T, double hz,
-                                          FaceCoef<NB>& f) {
+__device__ __forceinline__ void face_coef(const ImpecSide<NB>& c, const ImpecSide<NB>& n, bool z, bool minus, double T,
+                                          double hz, FaceCoef<NB>& f) {
   f.rs_up = 0.0;
 #pragma unroll
   for (int ph = 0; ph < NB; ++ph) {                // water, oil[, gas]
     double dphi = c.p[ph] - n.p[ph];
     if (z) dphi = fma(-(c.rho[ph] + n.rho[ph]), hz, dphi);
-    const bool up = nonneg(dphi);
+    const bool up = minus ? positive(dphi) : nonneg(dphi);
     f.c[ph] = T * sel(up, c.l[ph], n.l[ph]);
     f.dphi[ph] = dphi;
     if (ph == 1 && NB == 3) f.rs_up = sel(up, c.rs, n.rs);
@@ -202,7 +205,7 @@ __global__ void __launch_bounds__(32) impec_matrix_kernel(Params P, const double
       ImpecSide<NB> nb;
       impec_load<NB>(scratch + impec_at(n), z, nb);
       FaceCoef<NB> f;
-      face_coef<NB>(own, nb, z, trans[face], t == 0 ? P.grav_dz : -P.grav_dz, f);
+      face_coef<NB>(own, nb, z, t < 3, trans[face], t == 0 ? P.grav_dz : -P.grav_dz, f);
       // weights of the phase fluxes in the row: w_w, w_o + R_s w_g, w_g
       double a[NB];
       a[0] = f.c[0] * w[0];
@@ -264,7 +267,7 @@ __global__ void __launch_bounds__(64) impec_update_kernel(Params P, const double
     ImpecSide<NB> nb;
     impec_load<NB>(scratch + impec_at(n), z, nb);
     FaceCoef<NB> f;
-    face_coef<NB>(own, nb, z, trans[face], t == 0 ? P.grav_dz : -P.grav_dz, f);
+    face_coef<NB>(own, nb, z, t < 3, trans[face], t == 0 ? P.grav_dz : -P.grav_dz, f);
     const double dd = dpc - dp[n];
     // phase fluxes at the new pressure, then components (dissolved gas with the oil)
     double F[NB];
