@@ -536,7 +536,8 @@ __device__ __forceinline__ void masses(const Params& P, const Pvt& f, double p, 
   const double so = (NB == 3) ? (1.0 - sw - f.sg) : (1.0 - sw);
   const double O = phi * f.bo, mo = so * O;
   const double O_p = fma(phi_p, f.bo, phi * f.bo_p), mo_p = so * O_p;
-  const double mo_x = SAT ? neg(O) : fma(-f.sg_x, O, so * (phi * f.bo_x));
+  const double mo_q = SAT ? 0.0 : so * (phi * f.bo_x);      // the X derivative through b_o
+  const double mo_x = SAT ? neg(O) : fma(-f.sg_x, O, mo_q);
   if (PART != 1) {
     const double W = phi * f.bw;
     m[0] = sw * W;
@@ -556,7 +557,10 @@ __device__ __forceinline__ void masses(const Params& P, const Pvt& f, double p, 
     if (DERIV) {
       m_p[2] = fma(rso, O_p, fma(f.rs_p, mo, f.sg * fma(phi_p, f.bg, phi * f.bg_p)));
       m_sw[2] = -f.rs * O;
-      m_x[2] = SAT ? __dadd_rn(G, m_sw[2]) : fma(f.sg_x, G, fma(f.rs_x, mo, f.rs * mo_x));
+      // G - R_s O nearly cancels: its product is not rounded (rounded first, it
+      // took the entry's error from 2.6e-16 to 3.6e-16)
+      const double free = fma(-f.rs, O, G);
+      m_x[2] = SAT ? free : sel(nonzero(f.sg_x), free, fma(f.rs_x, mo, f.rs * mo_q));
     }
   }
 }
