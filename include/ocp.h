@@ -140,7 +140,7 @@ ocp_status ocp_linearize(ocp_grid* grid, const double* u_new, const int8_t* flag
  * application or framework with its own allocator, or a loop under a fixed
  * memory budget that may not grow.
  * Same arguments, outputs and errors as ocp_linearize, but its per-cell
- * scratch is a 32 MiB array owned by the library instead of the grid's
+ * scratch is a fixed array owned by the library instead of the grid's
  * buffer, so it accepts grids of at most 41 943 cells and returns
  * OCP_ERR_INVALID_ARG for larger ones.  It calls no cudaMalloc, cudaFree or
  * other allocating routine, and triggers no lazy module load: the array is

@@ -311,7 +311,7 @@ ocp_status ocp_impec_pressure(ocp_grid* g, const double* pn, double dt, double* 
   using namespace ocp;
   if (!g || !pn || !val || !rhs) return report(OCP_ERR_INVALID_ARG, "grid, pn, val and rhs are required");
   if (!(std::isfinite(dt) && dt > 0.0)) return report(OCP_ERR_INVALID_ARG, "dt must be finite and > 0");
-  static_assert(kImpecSlots <= 85, "IMPEC data must fit the linearisation scratch");
+  static_assert(kImpecSlots <= kScratchFields, "IMPEC data must fit the linearisation scratch");
   Guard guard(g->device);
   if (guard.err != cudaSuccess) return report(OCP_ERR_CUDA, "cudaSetDevice: %s", cudaGetErrorString(guard.err));
   cudaStream_t s = (cudaStream_t)stream;

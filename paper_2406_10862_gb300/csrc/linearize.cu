@@ -48,6 +48,7 @@ constexpr int kSelf = 25;   // own residual (3) + diagonal (9)   25 .. 36
 constexpr int kPart = 25;   // the same after the + faces, in their place
 constexpr int kInc = 37;    // shares handed over, 3 x (F 3 + dj 9)   37 .. 72
 constexpr int kFields = 73;
+static_assert(kFields == kScratchFields, "the grid's scratch holds one layout");
 // A cell's scratch: field f is at cell_scratch(scr, c)[32 * f].
 __device__ __forceinline__ double* cell_scratch(double* scr, long long c) {
   return scr + ((c >> 5) * (32 * kFields) + (c & 31));
@@ -1523,12 +1524,8 @@ cudaError_t preload_linearize(int nb) {
   return e;
 }
 
-// kFields doubles per cell, in whole tiles of 32 cells; 100 per cell are
-// reserved (the IMPEC path keeps its own layout in them).
-int64_t linearize_scratch_doubles(int64_t N) {
-  const int64_t tiles = (N + 31) / 32 * 32 * kFields;
-  return tiles > 100 * N ? tiles : 100 * N;
-}
+// Whole tiles of 32 cells (the IMPEC path keeps its own, smaller layout in them).
+int64_t linearize_scratch_doubles(int64_t N) { return (N + 31) / 32 * 32 * kScratchFields; }
 
 cudaError_t launch_linearize(const ocp_grid* g, const double* u_new, const int8_t* f_new,
                              const double* u_old, const int8_t* f_old, double dt, double* res,

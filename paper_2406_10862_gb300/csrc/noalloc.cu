@@ -8,9 +8,8 @@
 // inputs and outputs; this entry point itself calls no cudaMalloc, cudaFree
 // or any allocating routine.
 //
-// The array holds kStaticScratchDoubles doubles (32 MiB).  The scratch needs
-// 100 doubles per cell, so grids of at most kStaticScratchDoubles / 100 =
-// 41 943 cells are accepted; larger grids are rejected with
+// The array holds the scratch of kStaticScratchCells = 41 943 cells (24.5 MB, 73
+// doubles per cell in whole tiles of 32 cells); larger grids are rejected with
 // OCP_ERR_INVALID_ARG.
 //
 // When the array is reserved: with CUDA's lazy module loading (the default)
@@ -18,7 +17,7 @@
 // used there, and loading them allocates device memory.  So ocp_grid_create,
 // which allocates anyway, does that first use: on the grid's device it looks
 // up the array's device address with cudaGetSymbolAddress (which loads the
-// array, reserving its 32 MiB on that device until the process exits) and
+// array, reserving its memory on that device until the process exits) and
 // loads the linearisation kernels, and it keeps the address in the grid.  In
 // host code the array's name is only a host-side stand-in, never a device
 // address; device code could name it directly, host code uses the address.
@@ -36,9 +35,9 @@
 
 namespace {
 
-constexpr long long kStaticScratchDoubles = 4LL * 1024 * 1024;   // 32 MiB
+constexpr long long kStaticScratchCells = 41943;
 
-static __device__ __align__(256) double g_static_scratch[kStaticScratchDoubles];
+static __device__ __align__(256) double g_static_scratch[(kStaticScratchCells + 31) / 32 * 32 * ocp::kScratchFields];
 
 }  // namespace
 
@@ -65,11 +64,10 @@ extern "C" ocp_status ocp_linearize_noalloc(ocp_grid* g, const double* u_new, co
   if (g->prm.nb == 3 && (!flag_new || !flag_old))
     return ocp::report(OCP_ERR_INVALID_ARG, "flags are required with three phases");
   if (!(std::isfinite(dt) && dt > 0.0)) return ocp::report(OCP_ERR_INVALID_ARG, "dt must be finite and > 0");
-  const long long need = ocp::linearize_scratch_doubles(g->prm.N);
-  if (need > kStaticScratchDoubles)
+  if (g->prm.N > kStaticScratchCells)
     return ocp::report(OCP_ERR_INVALID_ARG,
                        "ocp_linearize_noalloc: grid has %lld cells but the static scratch holds at most %lld cells",
-                       (long long)g->prm.N, kStaticScratchDoubles / (need / g->prm.N));
+                       (long long)g->prm.N, kStaticScratchCells);
   if (!g->d_static_scratch)
     return ocp::report(OCP_ERR_CUDA, "ocp_linearize_noalloc: no device address for the static scratch");
 

@@ -19,6 +19,7 @@
 namespace ocp {
 
 constexpr int kMaxRows = 64;           // PVT table rows
+constexpr int kScratchFields = 73;     // doubles per cell of a grid's scratch, in whole tiles of 32 cells
 constexpr double kRbFt3 = 5.614583;    // ft^3 per reservoir barrel
 constexpr double kDarcy = 0.001127;    // rb cP / (day psi mD ft)
 constexpr double kGrav = 1.0 / 144.0;  // psi per (lb/ft^3 ft)
