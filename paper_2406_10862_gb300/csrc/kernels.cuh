@@ -23,6 +23,15 @@ cudaError_t static_scratch_address(double** out);
 cudaError_t preload_linearize(int nb);
 cudaError_t launch_perf_wi(ocp_grid* g, const double* lnk, cudaStream_t s);
 int64_t solver_work_doubles(const ocp_grid* g);
+// Places in the solver's work buffer, in doubles, for n unknowns in blocks of nb:
+// the six vectors r, v, p, s, r0, t, the scaled well columns, the block inverses
+// (used without the copy of the matrix) and the right-hand side without the
+// well unknowns.  The size told to callers is what it was when the reductions
+// had a vector and 633 partial sums in it: n + 633 doubles to spare.
+struct SolverWork {
+  int64_t wb, dinv, reduced, size;
+  SolverWork(int64_t nb, int64_t n) : wb(6 * n), dinv(7 * n), reduced((7 + nb) * n), size((9 + nb) * n + 633) {}
+};
 
 // Well terms of a Jacobian with bottom-hole-pressure unknowns, oriented for
 // the system being solved: bs couples the wells into the cell rows, cs the

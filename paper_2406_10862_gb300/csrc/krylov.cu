@@ -45,7 +45,9 @@ namespace {
 constexpr int kSolveThreads = 512;     // 128 registers a thread: a row's 36 loads in flight
 constexpr int kMinRange = 128;         // unknowns of a CTA at least: one warp per sub-partition
 constexpr int kMaxCtas = 256;
-constexpr int kVecs = 7;               // r, r0, p, v, s, t, x
+// The vectors, those that shared memory keeps longest first; x is the caller's,
+// the others stand in this order in the work buffer.
+enum { kR = 0, kV, kP, kS, kR0, kT, kX, kVecs };
 constexpr unsigned kSpin = 1u << 21;   // polls of one slot, above a second
 constexpr int kSmemVecBytes = 213 * 1024;
 // A copy of the scaled matrix of at most so many doubles (1 MiB: 2427 cells
@@ -80,7 +82,7 @@ struct SolveArgs {
   const double* val;                   // without planes: the matrix and the block inverses
   const double* dinv;
   int trans;
-  double* vec[kVecs];                  // r (holding D^-1 b at the start), r0, p, v, s, t, x
+  double* vec[kVecs];                  // kR holds D^-1 b at the start
   const int32_t* perf_of_cell;         // wells: perforations, D^-1 B / d and C
   const Perf* perf;
   const int32_t* first;
@@ -566,10 +568,9 @@ __global__ void __launch_bounds__(kSolveThreads, 1) solve_kernel(const __grid_co
   double* own[kVecs];
 #pragma unroll
   for (int q = 0; q < kVecs; ++q) own[q] = q < A.smem_vecs ? dyn + (long long)q * A.range : A.vec[q] + base;
-  // order of the vectors in shared memory: those read most often first
-  double *r = own[0], *v = own[1], *p = own[2], *s = own[3], *r0 = own[4], *t = own[5], *x = own[6];
-  double *pub_p = A.vec[2] + base, *pub_s = A.vec[3] + base;
-  const bool sm_p = A.smem_vecs > 2, sm_s = A.smem_vecs > 3;
+  double *r = own[kR], *v = own[kV], *p = own[kP], *s = own[kS], *r0 = own[kR0], *t = own[kT], *x = own[kX];
+  double *pub_p = A.vec[kP] + base, *pub_s = A.vec[kS] + base;
+  const bool sm_p = A.smem_vecs > kP, sm_s = A.smem_vecs > kS;
   unsigned long long epoch = A.epoch;
   double part[3] = {0.0, 0.0, 0.0};
   // no CTA's shared memory is written before the CTA runs
@@ -604,14 +605,14 @@ __global__ void __launch_bounds__(kSolveThreads, 1) solve_kernel(const __grid_co
       if (live) use(l, acc);
     }
   };
-  // y = D^-1 b stands in vec[0]; r0 = p = r = y - M x
-  apply(A.vec[6], nullptr, [&](int l, double m) {
-    const double y = A.vec[0][base + l], ri = y - m;
+  // y = D^-1 b stands in r's place; r0 = p = r = y - M x
+  apply(A.vec[kX], nullptr, [&](int l, double m) {
+    const double y = A.vec[kR][base + l], ri = y - m;
     r[l] = ri;
     r0[l] = ri;
     p[l] = ri;
     if (sm_p) pub_p[l] = ri;
-    if (A.smem_vecs > 6) x[l] = A.vec[6][base + l];
+    if (A.smem_vecs > kX) x[l] = A.vec[kX][base + l];
     part[0] = fma(y, y, part[0]);
     part[1] = fma(ri, ri, part[1]);
   });
@@ -628,7 +629,7 @@ __global__ void __launch_bounds__(kSolveThreads, 1) solve_kernel(const __grid_co
   apply_near(p, v);
   while (go) {
     // v = M p, then alpha and the test on r . r
-    apply(A.vec[2], v, [&](int l, double vi) {
+    apply(A.vec[kP], v, [&](int l, double vi) {
       v[l] = vi;
       part[0] = fma(r0[l], vi, part[0]);
     });
@@ -660,7 +661,7 @@ __global__ void __launch_bounds__(kSolveThreads, 1) solve_kernel(const __grid_co
     if (!grid_wait<0, true, CLUSTER>(A, sh, epoch)) return;
     // t = M s, then omega and rho
     part[0] = part[1] = part[2] = 0.0;
-    apply(A.vec[3], t, [&](int l, double ti) {
+    apply(A.vec[kS], t, [&](int l, double ti) {
       t[l] = ti;
       part[0] = fma(ti, s[l], part[0]);
       part[1] = fma(ti, ti, part[1]);
@@ -700,8 +701,8 @@ __global__ void __launch_bounds__(kSolveThreads, 1) solve_kernel(const __grid_co
     apply_near(p, v);
     if (!grid_wait<0, true, CLUSTER>(A, sh, epoch)) return;
   }
-  if (A.smem_vecs > 6)
-    for (int l = tid; l < len; l += T) A.vec[6][base + l] = x[l];
+  if (A.smem_vecs > kX)
+    for (int l = tid; l < len; l += T) A.vec[kX][base + l] = x[l];
   if (blockIdx.x == 0 && tid == 0) {
     A.result->iterations = (double)iter;
     A.result->rr = rr;
@@ -798,10 +799,7 @@ size_t solver_own_bytes(const ocp_grid* g) {
 }
 
 int64_t solver_work_doubles(const ocp_grid* g) {
-  const int64_t n = (int64_t)g->prm.nb * g->prm.N;
-  // r, r0, p, v, s, t; the scaled well columns; the block inverses (used
-  // without planes); and the reduced right-hand side of the well elimination
-  return 9 * n + (int64_t)g->prm.nb * g->prm.nb * g->prm.N + 633;
+  return SolverWork(g->prm.nb, g->prm.nb * g->prm.N).size;
 }
 
 void free_planes(ocp_grid* g) {
@@ -862,15 +860,15 @@ ocp_status bicgstab_run(ocp_grid* g, const double* val, const WellSchur* ws, con
   };
   A.planes = planes;
   A.val = val;
-  A.dinv = work + 8 * n;
+  const SolverWork place(nb, n);
+  A.dinv = work + place.dinv;
   A.trans = transpose ? 1 : 0;
-  // own[] order in solve_kernel: r, v, p, s, r0, t, x
-  for (int q = 0; q < kVecs - 1; ++q) A.vec[q] = work + q * n;
-  A.vec[6] = x;
+  for (int q = 0; q < kX; ++q) A.vec[q] = work + q * n;
+  A.vec[kX] = x;
   A.perf_of_cell = g->d_perf_of_cell;
   A.perf = g->d_perf;
   A.first = g->d_well_first;
-  double* wb = work + 7 * n;
+  double* wb = work + place.wb;
   A.wb = wb;
   A.wc = ws ? ws->cs : nullptr;
   A.rtol = rtol;
@@ -884,11 +882,11 @@ ocp_status bicgstab_run(ocp_grid* g, const double* val, const WellSchur* ws, con
   const WellSchur wsv = ws ? *ws : WellSchur{nullptr, nullptr, nullptr};
   if (e == cudaSuccess) e = cudaMemsetAsync(g->d_solve_sync, 0, sizeof(SolveResult), s);
   const unsigned blocks = (unsigned)((n + 255) / 256);
-  double* dinv = planes ? nullptr : work + 8 * n;
+  double* dinv = planes ? nullptr : work + place.dinv;
   auto scale = nb == 3 ? scale_kernel<3> : (nb == 2 ? scale_kernel<2> : scale_kernel<1>);
   if (e == cudaSuccess)
     e = launch_pdl(scale, blocks, 256, 0, s, g->prm, (int)n, val, A.trans, (const int32_t*)g->d_perf_of_cell,
-                   (const Perf*)g->d_perf, wsv, b, planes, dinv, A.vec[0], wb, g->d_status);
+                   (const Perf*)g->d_perf, wsv, b, planes, dinv, A.vec[kR], wb, g->d_status);
   void* args[] = {&A};
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];

@@ -1450,7 +1450,6 @@ ModelArgs model_args(const ocp_grid* g, double* scratch, const double* u_new, co
   M.P = g->prm;
   M.table = g->d_table;
   M.trans = g->d_trans;
-  M.row_ptr = g->d_row_ptr;
   M.phi = g->d_phi;
   M.perf_of_cell = g->d_perf_of_cell;
   M.perf = g->d_perf;

@@ -166,7 +166,6 @@ struct ModelArgs {
   Params P;
   const Table* table;
   const double* trans;
-  const int32_t* row_ptr;
   const double* phi;
   const int32_t* perf_of_cell;
   const Perf* perf;

@@ -97,8 +97,7 @@ constexpr int kSpmvThreads = 32;
 constexpr int kSpmvMinBlocks = 24;
 
 template <int NB>
-__global__ void __launch_bounds__(kSpmvThreads, kSpmvMinBlocks) spmv_grid_kernel(Params P, const int32_t* __restrict__ row_ptr,
-                                                        const double* __restrict__ val, double alpha,
+__global__ void __launch_bounds__(kSpmvThreads, kSpmvMinBlocks) spmv_grid_kernel(Params P, const double* __restrict__ val, double alpha,
                                                         const double* __restrict__ x, double beta,
                                                         double* __restrict__ y, int mode) {
   constexpr int B2 = NB * NB;
@@ -503,11 +502,11 @@ cudaError_t launch_spmv(const ocp_grid* g, const double* val, double alpha, cons
   const unsigned bblocks = (unsigned)((N + kBulkRows - 1) / kBulkRows);
   if (g->prm.nb == 3) {
     if (transpose) return launch_pdl(spmv_grid_t_kernel<3>, gblocks, kSpmvThreads, 0, s, g->prm, val, alpha, x, beta, y, mode);
-    return launch_pdl(spmv_grid_kernel<3>, gblocks, kSpmvThreads, 0, s, g->prm, (const int32_t*)g->d_row_ptr, val, alpha, x, beta, y, mode);
+    return launch_pdl(spmv_grid_kernel<3>, gblocks, kSpmvThreads, 0, s, g->prm, val, alpha, x, beta, y, mode);
   }
   if (transpose) return launch_pdl(spmv_grid_t_kernel<2>, gblocks, kSpmvThreads, 0, s, g->prm, val, alpha, x, beta, y, mode);
   if (bulk) return launch_pdl(spmv_bulk_kernel<2>, bblocks, kBulkRows, bulk_smem_bytes<2>(), s, g->prm, (long long)g->nnzb, val, alpha, x, beta, y, mode, g->d_status);
-  return launch_pdl(spmv_grid_kernel<2>, gblocks, kSpmvThreads, 0, s, g->prm, (const int32_t*)g->d_row_ptr, val, alpha, x, beta, y, mode);
+  return launch_pdl(spmv_grid_kernel<2>, gblocks, kSpmvThreads, 0, s, g->prm, val, alpha, x, beta, y, mode);
 }
 
 cudaError_t launch_vjp(const ocp_grid* g, const double* u_new, const int8_t* f_new, const double* u_old,

@@ -282,7 +282,7 @@ ocp_status ocp_bicgstab_wells(ocp_grid* g, const double* val, const double* well
   const long long n = (long long)g->prm.nb * g->prm.N;
   // transposed system [A^T C^T; B^T D]: the same elimination with B and C exchanged
   WellSchur ws{transpose ? well_c : well_b, transpose ? well_b : well_c, well_d};
-  double* bred = work + (solver_work_doubles(g) - n);
+  double* bred = work + SolverWork(g->prm.nb, n).reduced;
   cudaError_t e = cudaMemcpyAsync(bred, b, sizeof(double) * n, cudaMemcpyDeviceToDevice, s);
   // b' = b - B D^-1 b_w
   if (e == cudaSuccess) e = launch_well_reduce(g, ws, b_w, bred, s);

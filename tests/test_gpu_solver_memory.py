@@ -150,3 +150,31 @@ def test_the_c_interface_lends_refuses_and_releases():
     assert lend(None, 5) == O.OCP_ERR_INVALID_ARG and lend(buf, -1) == O.OCP_ERR_INVALID_ARG
     assert lib.ocp_solver_lend(None, None, 0) == O.OCP_ERR_INVALID_ARG
     assert lib.ocp_solver_release(None) == O.OCP_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("copy", [True, False])
+@pytest.mark.parametrize("dims", [(5, 4, 3), (17, 19, 13)])
+def test_the_work_buffer_is_not_overrun(monkeypatch, dims, copy):
+    need_gpu()
+    from paper_2406_10862_gb300 import ocp as O
+
+    _, _, val, b = _system(dims)
+    g, _ = W.tiny(*dims, wells=False)
+    g.wells = [W.Well(kind=0, phase=0, p_bh=4600.0, cells=np.arange(g.N))]     # every cell perforated
+    grid = O.Grid(g)
+    n, guard = grid.solver_work().numel(), 3.5
+    work = torch.full((n + 2,), guard, dtype=torch.float64, device="cuda")
+    rng = np.random.default_rng(0)
+    T = lambda a: torch.as_tensor(a, device="cuda")
+    wb, wc = T(0.01 * rng.normal(size=b.numel())), T(0.01 * rng.normal(size=b.numel()))
+    x, xw = torch.zeros_like(b), torch.zeros(1, dtype=torch.float64, device="cuda")
+    if not copy:
+        _refuse(monkeypatch, grid)
+    with warnings.catch_warnings():
+        warnings.simplefilter("ignore")
+        grid.bicgstab_wells(val, wb, wc, T(np.array([30.0])), b, T(np.array([1.0])), x, xw, RTOL, 2000,
+                            work=work[1:-1])
+    assert work[0] == guard and work[-1] == guard
+    z = grid.spmv(val, x) + wb * xw - b
+    assert float(z.norm()) < 1e-9 * float(b.norm())
+    assert abs(float(wc @ x + 30.0 * xw - 1.0)) < 1e-9
