@@ -237,17 +237,19 @@ __device__ __forceinline__ void cell_ijk(const Params& P, long long c, int& i, i
 // Number of stored blocks in the rows before cell c = (i, j, k): 7 per
 // earlier cell minus the missing neighbours of every earlier cell, in
 // closed form.  Block indices fit 32 bits (ocp_grid_create rejects 7 N >=
-// 2^31), where an add is one instruction instead of two.
+// 2^31), where an add is one instruction instead of two; I = long long where
+// the kernel is faster with the longer form.
+template <typename I = int>
 __device__ __forceinline__ long long row_start_ijk(const Params& P, long long c, int i, int j, int k) {
-  const int nx = P.nx, nxy = (int)P.nxy, N = (int)P.N, ci = (int)c;
-  const int q = k * P.ny + j;                    // c / nx
-  const int i0 = q + (i > 0);                    // earlier cells with i == 0
-  const int iL = q;                              // ... with i == nx-1
-  const int rem = j * nx + i;                    // c % nxy
-  const int j0 = k * nx + min(rem, nx);          // ... with j == 0
-  const int jL = k * nx + max(rem - (nxy - nx), 0);
-  const int k0 = min(ci, nxy);                   // ... with k == 0
-  const int kL = max(ci - (N - nxy), 0);         // ... with k == nz-1
+  const I nx = P.nx, nxy = (I)P.nxy, N = (I)P.N, ci = (I)c;
+  const I q = (I)k * P.ny + j;                 // c / nx
+  const I i0 = q + (i > 0);                    // earlier cells with i == 0
+  const I iL = q;                              // ... with i == nx-1
+  const I rem = (I)j * nx + i;                 // c % nxy
+  const I j0 = k * nx + min(rem, nx);          // ... with j == 0
+  const I jL = k * nx + max(rem - (nxy - nx), (I)0);
+  const I k0 = min(ci, nxy);                   // ... with k == 0
+  const I kL = max(ci - (N - nxy), (I)0);      // ... with k == nz-1
   return (long long)(7 * ci - (i0 + iL + j0 + jL + k0 + kL));
 }
 

@@ -16,6 +16,8 @@
 //                   and the block-CSR pattern.
 // well_rate_kernel  surface rates of each well (one thread per well, its
 //                   perforations summed in order).
+#include <type_traits>
+
 #include "block_io.cuh"
 #include "kernels.cuh"
 #include "ocp_internal.cuh"
@@ -155,8 +157,10 @@ __global__ void __launch_bounds__(kSpmvThreads, kSpmvMinBlocks) spmv_grid_kernel
 // wide load where it is aligned (1 122 000 rows 72.7 -> 63.8 us); the nine
 // loads of a 3x3 block hit L1 after the first, and bringing them through
 // shared memory in block order, as the linearisation stores them, measured
-// slower (200 000 rows 29.0 against 26.1 us).
-template <int NB>
+// slower (200 000 rows 29.0 against 26.1 us).  I: the type of the row starts; the
+// 3x3 product is faster with 64 bits (30 000 rows 5.47 against 5.76 us), the
+// adjoint with 32 (18.0 against 18.7).
+template <int NB, typename I = int>
 __device__ __forceinline__ void column_product(const Params& P, long long c, const double* __restrict__ val,
                                                const double* __restrict__ x, double (&acc)[NB]) {
   constexpr int B2 = NB * NB;
@@ -176,7 +180,7 @@ __device__ __forceinline__ void column_product(const Params& P, long long c, con
     int sn = 0;
 #pragma unroll
     for (int u = 0; u < 6 - t; ++u) sn += hn[u];
-    const double* blk = val + (row_start_ijk(P, n, ni, nj, nk) + sn) * B2;
+    const double* blk = val + (row_start_ijk<I>(P, n, ni, nj, nk) + sn) * B2;
     double b[B2];
     if constexpr (NB == 2) {
       load4_const(blk, b);
@@ -202,7 +206,7 @@ __global__ void __launch_bounds__(kSpmvThreads) spmv_grid_t_kernel(Params P, con
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c >= P.N) return;
   double acc[NB];
-  column_product<NB>(P, c, val, x, acc);
+  column_product<NB, std::conditional_t<NB == 3, long long, int>>(P, c, val, x, acc);
 #pragma unroll
   for (int v = 0; v < NB; ++v) {
     double o = acc[v];
