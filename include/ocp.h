@@ -3,7 +3,7 @@
  *
  * One fully implicit (FIM) Newton linearisation of the black-oil component
  * mass balances on a Cartesian grid with two-point fluxes, the block-CSR
- * matrix-vector product the linear solver iterates on, and the adjoint
+ * matrix-vector product that Krylov methods iterate on, and the adjoint
  * vector-Jacobian product.  The equations are the component conservation law
  * (eq. 1) with Darcy velocities (eq. 2) and the component amounts of eq. 4,
  * in the black-oil closure where saturations, compositions and densities
@@ -274,9 +274,9 @@ ocp_status ocp_batch_get_status(ocp_batch* batch, void* cuda_stream);
 
 /* Launch shape of ocp_linearize on one grid (for example one found by
  * ocp_batch_tune on a batch of that grid alone).  A new grid starts with one
- * CTA per tile, tiles of 64 cells for the cell stage and 32 for the face and
- * assembly stages; grids of fewer than 128 cells per SM start with ordered = 3,
- * and grids that fit one cluster (ocp_grid_cluster_tiles) with ordered = 4. */
+ * CTA per tile, tiles of 32 cells for the face and assembly stages and of 64 for
+ * the cell stage; grids of fewer than 128 cells per SM start with 32 there too
+ * and ordered = 3, and grids that fit one cluster (ocp_grid_cluster_tiles) with ordered = 4. */
 ocp_status ocp_grid_set_shape(ocp_grid* grid, const ocp_launch_shape* shape);
 /* The launch shape ocp_linearize currently uses on the grid. */
 ocp_status ocp_grid_get_shape(const ocp_grid* grid, ocp_launch_shape* shape);
@@ -301,15 +301,18 @@ int64_t ocp_solver_work_doubles(const ocp_grid* grid);
  * scaled cell by cell into the units of the unknowns.  x holds the initial guess
  * on entry and the solution on return; b and x are block-interleaved [nb*N]
  * device vectors; work is a device buffer of ocp_solver_work_doubles().
- * The iterations run in one cooperative launch with the convergence test on
- * the device; the stream is synchronised once, at the end.  The iteration reads
+ * The iterations run in one launch (a CTA on each of the stream's SMs, or one
+ * thread-block cluster for small systems) with the convergence test on the
+ * device; the stream is synchronised once, at the end.  The iteration reads
  * the solver's copy of D^-1 A (6 nb^2 doubles per cell, 6 for a scalar system) in
  * memory lent to the call (ocp_solver_lend), else in memory that the first call
  * allocates and the grid keeps until ocp_solver_release; where neither has room
  * for it, the same iteration runs, slower, from bsr_val itself.  Calls on one
- * grid must not overlap from several host threads.  The paper solves with CPR-preconditioned FGMRES in PETSc/Hypre
- * (Sec. 5.1); this plain Krylov solver serves the Newton, adjoint and test
- * drivers.  Returns OCP_ERR_TIMEOUT when maxit is reached, OCP_ERR_NONFINITE on breakdown;
+ * grid must not overlap from several host threads.  The paper solves with
+ * CPR-preconditioned FGMRES in PETSc/Hypre (Sec. 5.1); this plain Krylov solver
+ * serves the Newton, adjoint and test drivers.  Returns OCP_ERR_TIMEOUT when
+ * maxit is reached, or when a CTA's bounded wait for the others ran out (x is
+ * then undefined and the sticky status set), OCP_ERR_NONFINITE on breakdown;
  * *iters and *relres (may be NULL) report the final state. */
 ocp_status ocp_bicgstab(ocp_grid* grid, const double* bsr_val, const double* b, double* x, double rtol,
                         int maxit, int transpose, double* work, int* iters, double* relres, void* cuda_stream);

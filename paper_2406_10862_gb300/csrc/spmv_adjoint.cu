@@ -1,7 +1,8 @@
 // Block-CSR products and the adjoint vector-Jacobian product.
 //
 // spmv_grid_kernel  y = alpha A x + beta y on the grid's 7-point block pattern
-//                   (the kernel the linear solver iterates on, Sec. 3.3.3);
+//                   (Sec. 3.3.3; for callers' own Krylov methods, the
+//                   library's solver works on its scaled copy);
 // spmv_grid_t_kernel the transposed product: every output row gathers the
 //                   blocks (n, c) of its column, located in closed form, so
 //                   that it is owned by one thread and no atomics are needed;
