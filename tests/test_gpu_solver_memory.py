@@ -128,7 +128,12 @@ def test_the_c_interface_lends_refuses_and_releases():
     def lend(t, m):
         return lib.ocp_solver_lend(h, t.data_ptr() if t is not None else None, ctypes.c_int64(m))
 
-    free = lambda: torch.cuda.mem_get_info()[0]
+    free = lambda: torch.cuda.mem_get_info()[0] + torch.cuda.memory_reserved()
+    solve()                                      # loads both forms' kernels
+    assert lend(None, 0) == 0
+    solve()
+    _scaled_residual(grid, val, b, torch.zeros_like(b), False)
+    assert lib.ocp_solver_release(h) == 0
     assert lend(buf[1:], n) == 0
     before = free()
     st, want = solve()
